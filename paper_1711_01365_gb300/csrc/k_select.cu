@@ -1,87 +1,57 @@
-// Radix selection of the n_plus smallest (key, index) pairs, for the
-// volume-preserving step (Sec. 7: the n_plus points of largest dE take the
-// SO(n) class; the key is dE complemented so that smaller keys are larger dE,
-// and the grid index breaks ties, lower index first).  Twelve MSB-first passes
-// over 8-bit digits of the 96-bit composite (64-bit key, 32-bit index); each
-// pass histograms the digit among the points that match the prefix found so
-// far, and one thread picks the bucket that holds the remaining rank.
-#include "mbo_dev.cuh"
+// The passes after the first of the volume-preserving step's radix selection
+// (mbo_select.cuh; the first is fused with the keys, k_vp_delta).
+#include <algorithm>
+
+#include "mbo_select.cuh"
 
 namespace mbo {
 
-__device__ __forceinline__ unsigned digit_of(unsigned long long key, unsigned idx, int d) {
-  return d < 8 ? (unsigned)((key >> (56 - 8 * d)) & 0xffu) : ((idx >> (24 - 8 * (d - 8))) & 0xffu);
-}
-
-// The top 8*d bits of (key, idx) equal those of the prefix found so far.
-__device__ __forceinline__ bool prefix_match(unsigned long long key, unsigned idx,
-                                             unsigned long long hi, unsigned lo, int d) {
-  if (d == 0) return true;
-  if (d <= 8) {
-    const int sh = 64 - 8 * d;
-    return (key >> sh) == (hi >> sh);
-  }
-  if (key != hi) return false;
-  const int sh = 32 - 8 * (d - 8);
-  return (idx >> sh) == (lo >> sh);
-}
-
-// n >= 0: select n points; n < 0: select the count already in ss->n_plus.
-__global__ void k_select_init(SelectState* ss, long long n) {
-  if (threadIdx.x == 0) {
-    if (n >= 0) ss->n_plus = (unsigned long long)n;
-    ss->hi = 0;
-    ss->lo = 0;
-    ss->k = ss->n_plus;
-  }
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) ss->hist[i] = 0;
-}
-
-__global__ void __launch_bounds__(256)
-k_select_hist(const unsigned long long* __restrict__ keys, long long P, SelectState* ss, int d) {
-  __shared__ unsigned int h[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
-  __syncthreads();
-  const unsigned long long hi = ss->hi;
-  const unsigned lo = ss->lo;
-  if (ss->n_plus == 0) return;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < P;
-       x += (long long)gridDim.x * blockDim.x) {
+// Key digit d (1 .. 5), then index digits (d - 6) of an index of `bits` bits.
+__global__ void __launch_bounds__(kSelThreads)
+k_select_pass(const unsigned long long* __restrict__ keys, long long P, SelectState* ss, int d, int bits) {
+  __shared__ unsigned int h[kSelBins];
+  __shared__ unsigned int part[kSelThreads / 32];
+  __shared__ int s_flag;
+  if (ss->done) return;
+  const unsigned long long hi = ss->hi, k = ss->k;
+  const unsigned int lo = ss->lo;
+  sel_clear(h);
+  int sh, w;
+  const bool on_key = d < kSelKeyPasses;
+  if (on_key) key_digit(d, sh, w);
+  else idx_digit(bits, d - kSelKeyPasses, sh, w);
+  const unsigned int mask = (1u << w) - 1;
+  const int up = sh + w;  // <= 53 for a key digit, <= 32 for an index digit
+  const long long step = (long long)gridDim.x * kSelThreads;
+#pragma unroll 4
+  for (long long x = blockIdx.x * (long long)kSelThreads + threadIdx.x; x < P; x += step) {
     const unsigned long long key = keys[x];
-    if (prefix_match(key, (unsigned)x, hi, lo, d)) atomicAdd(&h[digit_of(key, (unsigned)x, d)], 1u);
+    if (on_key) {
+      if (key >> up == hi >> up) atomicAdd(&h[(unsigned)(key >> sh) & mask], 1u);
+    } else if (key == hi && (unsigned long long)x >> up == (unsigned long long)lo >> up) {
+      atomicAdd(&h[(unsigned)((unsigned)x >> sh) & mask], 1u);
+    }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    if (h[i]) atomicAdd(&ss->hist[i], h[i]);
+  if (!sel_flush(h, ss, &s_flag)) return;
+  int digit = 0;
+  unsigned long long rest = 0;
+  bool whole = false;
+  if (!sel_pick(ss, k, part, digit, rest, whole)) return;
+  if (on_key) {
+    sel_record_key(ss, hi, d, digit, rest, whole);
+  } else {
+    ss->lo = lo | (unsigned)digit << sh | (whole ? (1u << sh) - 1 : 0u);
+    ss->k = rest;
+    ss->done = whole ? 1 : 0;
+  }
 }
 
-__global__ void k_select_pick(SelectState* ss, int d) {
-  if (threadIdx.x != 0 || ss->n_plus == 0) return;
-  const unsigned long long k = ss->k;
-  unsigned long long cum = 0;
-  int b = 0;
-  for (; b < 255; ++b) {
-    const unsigned long long c = ss->hist[b];
-    if (cum + c >= k) break;
-    cum += c;
-  }
-  ss->k = k - cum;
-  if (d < 8) ss->hi |= ((unsigned long long)b) << (56 - 8 * d);
-  else ss->lo |= ((unsigned)b) << (24 - 8 * (d - 8));
-  for (int i = 0; i < 256; ++i) ss->hist[i] = 0;
-}
-
-cudaError_t launch_select(unsigned long long* keys, long long P, SelectState* ss, int blocks,
+cudaError_t launch_select(const unsigned long long* keys, long long P, SelectState* ss, int blocks,
                           cudaStream_t s) {
-  for (int d = 0; d < 12; ++d) {
-    k_select_hist<<<blocks, 256, 0, s>>>(keys, P, ss, d);
-    k_select_pick<<<1, 32, 0, s>>>(ss, d);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_select_init(SelectState* ss, long long n, cudaStream_t s) {
-  k_select_init<<<1, 256, 0, s>>>(ss, n);
+  int bits = 1;
+  while (bits < 32 && (1ll << bits) < P) ++bits;
+  const int passes = kSelKeyPasses + (bits + 10) / 11;
+  for (int d = 1; d < passes; ++d) k_select_pass<<<blocks, kSelThreads, 0, s>>>(keys, P, ss, d, bits);
   return cudaGetLastError();
 }
 

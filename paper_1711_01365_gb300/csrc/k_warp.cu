@@ -27,8 +27,9 @@ k_wrow(Geom g, Tables<float> t, const float* __restrict__ Ain, float* A, float2*
   constexpr int C = NM * NM, Q = (C + 1) / 2, E = F::E, RS = F::RS, NT = wrow_threads(N, NM);
   constexpr int PS = R * RS;  // slots of one (row, plane): R group regions, >= N
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double redd[32];
-  __shared__ int redi[32];
+  constexpr int NTS = wrow_threads(N, NM);
+  __shared__ double redd[MODE == ROW_FWD ? 32 : 1];
+  __shared__ StatsShared<float, MODE == ROW_INV_PROJECT_FWD ? NTS : 1> sh;
   __shared__ int s_flag, s_nfb;
   pdl_wait();  // the previous pass's spectrum and run state are complete
   if (sp.respect_stop && *(volatile int*)&sp.st->stop) return;
@@ -50,6 +51,7 @@ k_wrow(Geom g, Tables<float> t, const float* __restrict__ Ain, float* A, float2*
   const bool mirror = q == Q - 1 && g.xh < N;
   float2 v[E];
   PointStats<float> ps;  // projection mode: over all of the block's rows
+  bool last = false;     // projection mode, thread 0: this block arrived last
   double defect = 0.0;   // forward mode
 
   // Row groups of this block: its own index, or with PERS the groups
@@ -77,26 +79,34 @@ k_wrow(Geom g, Tables<float> t, const float* __restrict__ Ain, float* A, float2*
     };
 
     if (MODE == ROW_FWD) {
-      // per point: load all channels, accumulate n - |A|^2, park the planes
-      for (int p = tid; p < RB * N; p += NT) {
-        const int rw = p / N, x = p - rw * N;
-        if (row0 + rw >= rows) continue;
-        const long long o = (row0 + rw) * N + x;
-        float sq = 0.f;
+      // The rows straight into registers (one address per element, constant
+      // offsets): lane (q, r, l) takes channels 2q and 2q + 1 of its own points,
+      // so nothing is exchanged before the transform.  sum n - |A|^2: the plane
+      // that comes first brings the n of its points, every lane takes off its
+      // squares, summed in two FP32 words (TwoSum) and joined in FP64.
+      const float* a0 = Ain + (2 * q) * P + off + r;
+      const float* a1 = a0 + P;
+      const bool pair = 2 * q + 1 < C;
+      if (!live) {
 #pragma unroll
-        for (int qq = 0; qq < Q; ++qq) {
-          const float re = Ain[(2 * qq) * P + o];
-          const float im = (2 * qq + 1 < C) ? Ain[(2 * qq + 1) * P + o] : 0.f;
-          sm[(rw * Q + qq) * PS + x] = float2{re, im};
-          sq += re * re + im * im;
+        for (int j = 0; j < E; ++j) v[j] = float2{0.f, 0.f};
+      } else {
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[j].x = a0[R * (l + LQ * j)];
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[j].y = pair ? a1[R * (l + LQ * j)] : 0.f;
+        if (sp.do_stats) {
+          float hi = 0.f, lo = 0.f;
+#pragma unroll
+          for (int j = 0; j < E; ++j) {
+            const float t2 = v[j].x * v[j].x + v[j].y * v[j].y;
+            const float sm2 = hi + t2, bb = sm2 - hi;
+            lo += (hi - (sm2 - bb)) + (t2 - bb);
+            hi = sm2;
+          }
+          defect += ((q == 0 ? (double)(NM * E) : 0.0) - (double)hi) - (double)lo;
         }
-        defect += (double)(float(NM) - sq);
       }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < E; ++j) v[j] = base[R * (l + LQ * j) + r];
-      if constexpr (R > 1) __syncthreads();  // regions are shared across groups
-      else __syncwarp();
       F::fwd(v, base, r, tw, twr, l);
       store_spectrum(v);
       return;
@@ -222,7 +232,13 @@ k_wrow(Geom g, Tables<float> t, const float* __restrict__ Ain, float* A, float2*
         finish_point<NM>(A, P, ro, x, old, b, sg, sm + rw * Q * PS + x, PS, ps);
       }
     }
+    // one row group per block: its statistics are complete, and the arrival at
+    // the grid's counter overlaps the forward transform below (a block that
+    // walks several groups arrives after its loop: the test for the last one
+    // cost the 2048-point rows 1%)
+    if (!PERS && sp.do_stats) stats_park(ps, sh);
     __syncthreads();
+    if (!PERS && sp.do_stats) last = stats_arrive(sp, sh);
 #pragma unroll
     for (int j = 0; j < E; ++j) v[j] = base[R * (l + LQ * j) + r];
     if constexpr (R > 1) __syncthreads();
@@ -246,7 +262,12 @@ k_wrow(Geom g, Tables<float> t, const float* __restrict__ Ain, float* A, float2*
     if (grid_sum(tot, sp.rb, redd, &s_flag, &all) && tid == 0) sp.st->defect = all;
     return;
   }
-  finalize_step_stats(g.P, g.tau, sp, ps, redd, redi, &s_flag);
+  if constexpr (PERS) {
+    stats_park(ps, sh);
+    __syncthreads();
+    last = stats_arrive(sp, sh);
+  }
+  stats_finish(g.P, g.tau, sp, last, sh);
 }
 
 template <int NM, int MODE, int N>
@@ -276,7 +297,8 @@ cudaError_t wrow_nm(const Geom& g, const Tables<float>& t, const float* Ain, flo
   // a block prefetches the spectrum rows of the block one wave later
   const int ahead = blocks > resident ? resident : 0;
   // persistent: one wave of blocks walks the row groups with a stride of the grid
-  if (CAN_PERS && wrow_persistent_flag() && blocks > resident)
+  // (also wherever the last block would have too many records to sum)
+  if (CAN_PERS && blocks > resident && (wrow_persistent_flag() || blocks > (int)kReduceOneLevel))
     return launch_pdl(kp, resident, wrow_threads(N, NM), smem, s, g, t, Ain, A, static_cast<float2*>(W),
                       sp, fb, 0);
   return launch_pdl(k, blocks, wrow_threads(N, NM), smem, s, g, t, Ain, A, static_cast<float2*>(W), sp,

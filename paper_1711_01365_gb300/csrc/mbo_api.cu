@@ -18,6 +18,7 @@
 #include "../../include/mbo.h"
 #include "mbo_dev.cuh"
 #include "mbo_internal.h"
+#include "mbo_select.cuh"
 #include "mbo_tma.cuh"
 
 namespace mbo {
@@ -148,7 +149,9 @@ struct mbo_ctx {
   void* W = nullptr;
   void* tabs = nullptr;  // twiddles, multipliers (one allocation)
   size_t tabs_bytes = 0;
+  void* ctl = nullptr;        // one allocation for the arrays below
   double* part = nullptr;     // per-block partials, then per-group totals
+  BlockRecord* rec = nullptr; // per-block step statistics of the projecting passes
   double* epart = nullptr;    // per-block energy partials of the fused step's multiplier pass
   unsigned int* cnt = nullptr;  // per-group arrival counters + the group counter
   size_t ngroups = 0;
@@ -311,6 +314,7 @@ StatsPtrs stats_ptrs(mbo_ctx* h, bool stats, bool respect_stop, double tol) {
   sp.hist = h->hist;
   sp.rb.part = h->part;
   sp.rb.gpart = h->part + h->ngroups * kReduceGroup;
+  sp.rb.rec = h->rec;
   sp.rb.gcount = h->cnt;
   sp.rb.done = h->cnt + h->ngroups;
   sp.respect_stop = respect_stop ? 1 : 0;
@@ -662,11 +666,7 @@ mbo_status mbo_destroy(mbo_handle h) {
   if (h->cap) cudaStreamDestroy(h->cap);
   cudaFree(h->W);
   cudaFree(h->tabs);
-  cudaFree(h->part);
-  cudaFree(h->cnt);
-  cudaFree(h->st);
-  cudaFree(h->epart);
-  cudaFree(h->hist_mem);
+  cudaFree(h->ctl);
   cudaFree(h->field);
   cudaFree(h->vp_at);
   cudaFree(h->vp_keys);
@@ -807,15 +807,31 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
   const int tiles = g.Q * std::max(g.nz, g.ny) * (g.nx / min_tx);
   const size_t nparts = (size_t)std::max(rows, tiles);
   h->ngroups = (nparts + kReduceGroup - 1) / kReduceGroup;
-  if (!alloc(&h->W, wbytes) ||
-      !alloc((void**)&h->part, (h->ngroups * kReduceGroup + h->ngroups) * sizeof(double)) ||
-      !alloc((void**)&h->epart, h->ngroups * kReduceGroup * sizeof(double)) ||
-      !alloc((void**)&h->cnt, (h->ngroups + 1) * sizeof(unsigned int)) ||
-      !alloc((void**)&h->st, sizeof(RunState)) ||
-      !alloc(&h->hist_mem, (size_t)kRing * 5 * sizeof(double))) {
+  // the small control arrays share one allocation
+  size_t ctl_bytes = 0;
+  auto reserve = [&](size_t bytes) {
+    const size_t o = ctl_bytes;
+    ctl_bytes = (o + bytes + 255) & ~(size_t)255;
+    return o;
+  };
+  const size_t slots = h->ngroups * kReduceGroup;
+  const size_t o_st = reserve(sizeof(RunState)), o_cnt = reserve((h->ngroups + 1) * sizeof(unsigned int));
+  const size_t o_hist = reserve((size_t)kRing * 5 * sizeof(double));
+  const size_t zero_bytes = ctl_bytes;  // state, counters and records start at zero
+  const size_t o_part = reserve((slots + h->ngroups) * sizeof(double)), o_epart = reserve(slots * sizeof(double));
+  // records: grids of up to kReduceOneLevel blocks, or one wave (at most 32 blocks on each SM)
+  const size_t o_rec = reserve(std::min<size_t>(slots, 8192) * sizeof(BlockRecord));
+  if (!alloc(&h->W, wbytes) || !alloc(&h->ctl, ctl_bytes)) {
     mbo_destroy(h);
     return rc;
   }
+  char* ctl = static_cast<char*>(h->ctl);
+  h->st = reinterpret_cast<RunState*>(ctl + o_st);
+  h->cnt = reinterpret_cast<unsigned int*>(ctl + o_cnt);
+  h->hist_mem = ctl + o_hist;
+  h->part = reinterpret_cast<double*>(ctl + o_part);
+  h->epart = reinterpret_cast<double*>(ctl + o_epart);
+  h->rec = reinterpret_cast<BlockRecord*>(ctl + o_rec);
   char* hm = static_cast<char*>(h->hist_mem);
   h->hist.energy = reinterpret_cast<double*>(hm);
   h->hist.maxdelta = reinterpret_cast<double*>(hm + kRing * 8);
@@ -853,9 +869,7 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
       h->wmap_ok[ax] = true;
     }
   }
-  if (cudaMemset(h->st, 0, sizeof(RunState)) != cudaSuccess ||
-      cudaMemset(h->cnt, 0, (h->ngroups + 1) * sizeof(unsigned int)) != cudaSuccess ||
-      cudaMemset(h->hist_mem, 0, (size_t)kRing * 5 * sizeof(double)) != cudaSuccess ||
+  if (cudaMemset(h->ctl, 0, zero_bytes) != cudaSuccess ||
       cudaMallocHost((void**)&h->h_st, sizeof(RunState)) != cudaSuccess ||
       cudaMallocHost(&h->h_hist, (size_t)kRing * 5 * sizeof(double)) != cudaSuccess ||
       cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess) {
@@ -1170,26 +1184,34 @@ mbo_status mbo_profile_read(mbo_handle h, double* ms, int64_t* launches, int npa
 // Volume-preserving MBO (Sec. 7)
 // ---------------------------------------------------------------------------
 
-static mbo_status vp_buffers(mbo_handle h) {
-  if (h->vp_at) return MBO_OK;
+static mbo_status vp_buffers(mbo_handle h, cudaStream_t s) {
+  if (h->vp_ss) return MBO_OK;  // the last of them
   const size_t fbytes = (size_t)h->g.C * (size_t)h->g.P * h->elem;
-  CK(cudaMalloc(&h->vp_at, fbytes));
-  CK(cudaMalloc((void**)&h->vp_keys, (size_t)h->g.P * sizeof(unsigned long long)));
-  CK(cudaMalloc((void**)&h->vp_ss, sizeof(SelectState)));
+  if (!h->vp_at) CK(cudaMalloc(&h->vp_at, fbytes));
+  if (!h->vp_keys) CK(cudaMalloc((void**)&h->vp_keys, (size_t)h->g.P * sizeof(unsigned long long)));
+  SelectState* ss = nullptr;
+  CK(cudaMalloc((void**)&ss, sizeof(SelectState)));
+  const cudaError_t e = cudaMemsetAsync(ss, 0, sizeof(SelectState), s);
+  if (e != cudaSuccess) {
+    cudaFree(ss);
+    return fail(h, MBO_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+  }
+  h->vp_ss = ss;
   h->bytes_total += fbytes + (size_t)h->g.P * 8 + sizeof(SelectState);
   return MBO_OK;
 }
 
-static cudaError_t vp_launch(mbo_handle h, int which, const void* At, void* A, const StatsPtrs& sp,
-                             cudaStream_t s) {
+static cudaError_t vp_launch(mbo_handle h, VolumePass which, const void* At, void* A, const StatsPtrs& sp,
+                             cudaStream_t s, long long n_plus = 0) {
   long long blocks = (h->g.P + 255) / 256;
-  const long long cap = std::min<long long>((long long)h->ngroups * kReduceGroup, 152 * 16);
+  // eight blocks of 256 threads fit on an SM: one wave, one record per block
+  const long long cap = std::min<long long>((long long)h->ngroups * kReduceGroup, 152 * 8);
   if (blocks > cap) blocks = cap;
   if (h->dtype == MBO_F32)
     return launch_volume<float>(which, h->g, static_cast<const float*>(At), static_cast<float*>(A),
-                                h->vp_keys, h->vp_ss, sp, h->cfg.fallback_sigma, (int)blocks, s);
+                                h->vp_keys, h->vp_ss, sp, h->cfg.fallback_sigma, (int)blocks, s, n_plus);
   return launch_volume<double>(which, h->g, static_cast<const double*>(At), static_cast<double*>(A),
-                               h->vp_keys, h->vp_ss, sp, 0.0, (int)blocks, s);
+                               h->vp_keys, h->vp_ss, sp, 0.0, (int)blocks, s, n_plus);
 }
 
 // One volume-preserving step: diffuse (energy of A recorded), dE keys,
@@ -1202,15 +1224,10 @@ static mbo_status vp_step(mbo_handle h, void* A, long long n_plus, bool respect_
   CK(row_pass(h, ROW_FWD, A, nullptr, sp, s));
   CK(middle_passes(h, AXIS_FGI, sp, s));
   CK(row_pass(h, ROW_INV_OUT, nullptr, h->vp_at, none, s));
-  CK(vp_launch(h, 0, h->vp_at, A, none, s));
-  if (n_plus < 0) {
-    CK(cudaMemsetAsync(&h->vp_ss->n_plus, 0, sizeof(unsigned long long), s));
-    CK(vp_launch(h, 1, h->vp_at, A, none, s));
-  }
-  CK(launch_select_init(h->vp_ss, n_plus, s));
-  long long blocks = std::min<long long>((h->g.P + 255) / 256, 152 * 16);
+  CK(vp_launch(h, VP_DELTA_SELECT, h->vp_at, A, none, s, n_plus));
+  const long long blocks = std::min<long long>((h->g.P + kSelThreads - 1) / kSelThreads, 152 * 8);
   CK(launch_select(h->vp_keys, h->g.P, h->vp_ss, (int)blocks, s));
-  CK(vp_launch(h, 2, h->vp_at, A, sp, s));
+  CK(vp_launch(h, VP_ASSIGN, h->vp_at, A, sp, s));
   h->w_valid_for = nullptr;
   return MBO_OK;
 }
@@ -1222,8 +1239,8 @@ mbo_status mbo_step_volume(mbo_handle h, void* A, int64_t n_plus, mbo_stats* sta
   if ((rc = check_field_ptr(h, A, "A")) != MBO_OK) return rc;
   if (n_plus > h->g.P) return fail(h, MBO_ERR_INVALID_ARG, "n_plus exceeds the number of points");
   DeviceGuard dg(h->dev);
-  if ((rc = vp_buffers(h)) != MBO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if ((rc = vp_buffers(h, s)) != MBO_OK) return rc;
   if ((rc = vp_step(h, A, n_plus, false, -1.0, s)) != MBO_OK) return rc;
   if (stats) {
     CK(cudaStreamSynchronize(s));
@@ -1243,13 +1260,13 @@ mbo_status mbo_run_volume(mbo_handle h, void* A, int64_t n_plus, int max_steps, 
   if ((rc = check_field_ptr(h, A, "A")) != MBO_OK) return rc;
   if (n_plus > h->g.P) return fail(h, MBO_ERR_INVALID_ARG, "n_plus exceeds the number of points");
   DeviceGuard dg(h->dev);
-  if ((rc = vp_buffers(h)) != MBO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if ((rc = vp_buffers(h, s)) != MBO_OK) return rc;
   CK(cudaMemsetAsync(h->st, 0, sizeof(RunState), s));
   if (n_plus < 0) {  // fix the volume of the initial field once
     const StatsPtrs none = stats_ptrs(h, false, false, -1.0);
     CK(cudaMemsetAsync(&h->vp_ss->n_plus, 0, sizeof(unsigned long long), s));
-    CK(vp_launch(h, 1, nullptr, A, none, s));
+    CK(vp_launch(h, VP_COUNT, nullptr, A, none, s));
     unsigned long long cnt = 0;
     CK(cudaMemcpyAsync(&cnt, &h->vp_ss->n_plus, sizeof(cnt), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

@@ -1059,20 +1059,23 @@ template <typename T> __device__ T block_max(T v, T* red) {
   return r;
 }
 
+// One arrival at a device-scope counter, acquire-release: what this thread
+// wrote (and, past a block barrier, what its block wrote) is visible to
+// whoever sees the count, and the other way round.  Returns the count before.
+__device__ __forceinline__ unsigned int arrive_acq_rel(unsigned int* counter) {
+  unsigned int prev;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(counter) : "memory");
+  return prev;
+}
+
 // Arrival counter: returns true in exactly one of `expected` arriving blocks
 // (the last), after all of their earlier global writes are visible to it.
 __device__ __forceinline__ bool last_to_arrive(unsigned int* counter, unsigned int expected,
                                                int* s_flag) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int prev = atomicAdd(counter, 1u);
-    *s_flag = (prev == expected - 1) ? 1 : 0;
-  }
+  if (threadIdx.x == 0) *s_flag = (arrive_acq_rel(counter) == expected - 1) ? 1 : 0;
   __syncthreads();
-  const bool last = *s_flag != 0;
-  if (last) __threadfence();
-  return last;
+  return *s_flag != 0;
 }
 
 // Fixed-order sum of a partial array by one block (deterministic).
@@ -1080,35 +1083,6 @@ __device__ __forceinline__ double sum_partials(const double* p, int count, doubl
   double acc = 0.0;
   for (int i = threadIdx.x; i < count; i += blockDim.x) acc += __ldcg(&p[i]);
   return block_sum(acc, red);
-}
-
-// Two fixed-order partial sums by one block in one pass (their loads overlap):
-// the same per-thread split and reduction tree as sum_partials, so each total
-// is bit-identical to sum_partials of its array.  At most 16 warps; red needs
-// 32 slots.
-__device__ __forceinline__ void sum_partials2(const double* p1, int n1, const double* p2, int n2,
-                                              double* red, double& s1, double& s2) {
-  double a1 = 0.0, a2 = 0.0;
-  const int n = n1 > n2 ? n1 : n2;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    if (i < n1) a1 += __ldcg(&p1[i]);
-    if (i < n2) a2 += __ldcg(&p2[i]);
-  }
-  a1 = warp_sum(a1);
-  a2 = warp_sum(a2);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) {
-    red[w] = a1;
-    red[16 + w] = a2;
-  }
-  __syncthreads();
-  s1 = s2 = 0.0;
-  if (w == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    s1 = warp_sum((l < nw) ? red[l] : 0.0);
-    s2 = warp_sum((l < nw) ? red[16 + l] : 0.0);
-  }
 }
 
 // Deterministic grid-wide sum of one double per block (thread 0's v).  Up to
@@ -1119,20 +1093,15 @@ __device__ __forceinline__ void sum_partials2(const double* p1, int n1, const do
 // true in exactly one block, whose thread 0 receives the total.  The
 // counters return to zero.
 __device__ __forceinline__ bool grid_sum(double v, const ReduceBufs& rb, double* red, int* s_flag,
-                                         double* total, const double* extra = nullptr,
-                                         const unsigned* extra_n = nullptr, double* extra_total = nullptr) {
+                                         double* total) {
   const unsigned nb = gridDim.x, b = blockIdx.x;
   if (nb <= kReduceOneLevel) {
     // one level: the last block to arrive sums every partial in index order
-    // (and, when asked, another partial array in the same pass)
     if (threadIdx.x == 0) rb.part[b] = v;
     if (!last_to_arrive(&rb.gcount[0], nb, s_flag)) return false;
-    double t, te = 0.0;
-    if (extra) sum_partials2(rb.part, (int)nb, extra, (int)*extra_n, red, t, te);
-    else t = sum_partials(rb.part, (int)nb, red);
+    const double t = sum_partials(rb.part, (int)nb, red);
     if (threadIdx.x == 0) {
       *total = t;
-      if (extra) *extra_total = te;
       rb.gcount[0] = 0;
     }
     return true;
@@ -1149,10 +1118,8 @@ __device__ __forceinline__ bool grid_sum(double v, const ReduceBufs& rb, double*
   }
   if (!last_to_arrive(rb.done, ngroups, s_flag)) return false;
   const double t = sum_partials(rb.gpart, (int)ngroups, red);
-  const double te = extra ? sum_partials(extra, (int)*extra_n, red) : 0.0;
   if (threadIdx.x == 0) {
     *total = t;
-    if (extra) *extra_total = te;
     *rb.done = 0;
   }
   return true;

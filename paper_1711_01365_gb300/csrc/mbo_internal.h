@@ -51,13 +51,8 @@ struct Plan {
   Stage st[kMaxStages];
 };
 
-// Device-resident state of a run.  Accumulators are reset by the finaliser
-// of the projection pass at the end of every step.
+// Device-resident state of a run.
 struct RunState {
-  unsigned long long maxdelta_bits;  // bit pattern of a non-negative double (atomicMax)
-  unsigned long long flips;
-  unsigned long long fallback;
-  unsigned long long nonfinite;
   double defect;       // sum_x (n - |A(x)|_F^2) of the field whose spectrum is in the workspace
   double energy_last;  // last energy written by a transform pass
   long long step;      // steps completed in this run
@@ -145,8 +140,15 @@ enum RowMode { ROW_FWD = 0, ROW_INV_OUT = 1, ROW_INV_PROJECT_FWD = 2 };
 // Buffers of the deterministic two-level grid sum (see grid_sum).
 constexpr int kReduceGroup = 256;
 constexpr unsigned kReduceOneLevel = 2048;  // grids up to this size reduce in one level
+// Step statistics of one block besides its defect sum.
+struct alignas(16) BlockRecord {
+  unsigned long long maxd_bits;  // largest |delta|, the bits of a non-negative double
+  unsigned long long pad0_;
+  unsigned int flips, fallback, nonfinite, pad1_;  // one 16-byte load
+};
 struct ReduceBufs {
   double* part;          // one partial per block
+  BlockRecord* rec;      // one record per block (projecting passes)
   double* gpart;         // one total per group of kReduceGroup blocks
   unsigned int* gcount;  // arrivals per group (zero between launches)
   unsigned int* done;    // groups finished (zero between launches)
@@ -169,20 +171,27 @@ struct StatsPtrs {
 };
 
 // Radix selection of the n_plus smallest (key, index) pairs (volume-preserving
-// step).  After the passes, (hi, lo) is the n_plus-th smallest pair; a point is
-// selected iff (key, index) <= (hi, lo) and n_plus > 0.
+// step, mbo_select.cuh).  After the passes a point is selected iff (key, index)
+// <= (hi, lo) and n_plus > 0.  hist, count and positive are zero between steps
+// (zeroed at allocation; every step leaves them so).
+constexpr int kSelBins = 2048;
 struct SelectState {
-  unsigned long long hi;     // key part of the prefix / result
-  unsigned int lo;           // index part
+  unsigned long long hi;        // key part of the prefix / result
+  unsigned int lo;              // index part
+  int done;                     // the threshold is known: the passes that follow return
+  unsigned long long k;         // remaining rank (1-based) inside the current prefix
+  unsigned long long n_plus;    // points to select
+  unsigned long long positive;  // points with det > 0 (counted where n_plus is not given)
+  unsigned int count;           // blocks that finished the current pass
   unsigned int pad_;
-  unsigned long long k;      // remaining rank (1-based) inside the current prefix
-  unsigned long long n_plus; // points to select
-  unsigned int hist[256];
+  unsigned int hist[kSelBins];
 };
 
-cudaError_t launch_select(unsigned long long* keys, long long P, SelectState* ss, int blocks,
+// Which kernels launch_volume launches.
+enum VolumePass { VP_DELTA = 0, VP_COUNT = 1, VP_ASSIGN = 2, VP_DELTA_SELECT = 3 };
+
+cudaError_t launch_select(const unsigned long long* keys, long long P, SelectState* ss, int blocks,
                           cudaStream_t s);
-cudaError_t launch_select_init(SelectState* ss, long long n, cudaStream_t s);
 
 // Launchers (defined per element type in k_f32.cu / k_f64.cu).
 template <typename R>
@@ -232,9 +241,9 @@ bool wcol_tensor_map(CUtensorMap* map, void* W, const Geom& g, int axis, int tx)
 template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>& t, int tx,
                                                   int stages);
 template <typename R>
-cudaError_t launch_volume(int which, const Geom& g, const R* At, R* A, unsigned long long* keys,
+cudaError_t launch_volume(VolumePass which, const Geom& g, const R* At, R* A, unsigned long long* keys,
                           SelectState* ss, const StatsPtrs& sp, double fb, int blocks,
-                          cudaStream_t s);
+                          cudaStream_t s, long long n_plus = 0);
 
 // Replace the per-axis multipliers of a handle's diffusion (mbo_api.cu).
 // mult[ax] (ax = 0: x, 1: y, 2: z; z ignored in 2-D) holds N_ax values in

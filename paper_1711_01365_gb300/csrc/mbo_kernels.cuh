@@ -20,7 +20,11 @@
 //                 new field for the next step
 // 3-D adds k_axis<FWD> and k_axis<INV> along y around the z pass.
 #pragma once
+#include <algorithm>
+#include <atomic>
+
 #include "mbo_dev.cuh"
+#include "mbo_select.cuh"
 
 namespace mbo {
 
@@ -175,88 +179,158 @@ __device__ __forceinline__ void finish_point(R* __restrict__ A, long long P, lon
   for (int q = 0; q < Q; ++q) dst[q * qstride] = V{b[2 * q], (2 * q + 1 < C) ? b[2 * q + 1] : R(0)};
 }
 
-// Reduce a block's point statistics and, in the last block of the grid,
-// record the step (energy slot filled earlier by the transform pass; max
-// delta, flips, re-projections, non-finite count), decide stationarity
-// (tol >= 0), reset the accumulators and advance the step counter.
-template <typename R>
-__device__ __forceinline__ void finalize_step_stats(long long P, double tau, const StatsPtrs& sp,
-                                                    const PointStats<R>& ps, double* redd, int* redi,
-                                                    int* s_flag) {
+// Step statistics of a projecting pass, in three parts, so that the arrival at
+// the grid's counter overlaps the forward transform that follows the
+// projection:
+//   stats_park    every thread, before a block barrier: the largest change and
+//                 the counts are folded over the warp in integer instructions
+//                 (the bits of non-negative floats order like the floats), the
+//                 defects are parked in shared memory;
+//   stats_arrive  warp 0, after that barrier: sums the parked defects in FP64,
+//                 writes the block's record and arrives at the counter;
+//   stats_finish  every thread, at the end: the last block to have arrived
+//                 reduces all records in block order and records the step.
+// FP64 runs at 1/64 of the FP32 rate here (a warp-wide FP64 add holds the SM's
+// FP64 pipe for 16 cycles), so a butterfly of FP64 sums and maxima in every
+// warp was the expensive part: one warp per block does it now, for the defects
+// only.  The counter is one acquire-release atomic instead of a sequentially
+// consistent fence, an atomicMax and a relaxed counter.
+template <typename R, int NT> struct StatsShared {
+  R defect[NT];
+  unsigned long long maxd[16];
+  unsigned int cnt[3][16];
+  double sum[2][16];
+  int last;
+};
+
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
+    v = w > v ? w : v;
+  }
+  return v;
+}
+
+template <typename R, int NT>
+__device__ __forceinline__ void stats_park(const PointStats<R>& ps, StatsShared<R, NT>& sh) {
   const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
-  // one fused block reduction (blocks of at most 16 warps): the defect sum,
-  // the largest change, and the three counts in 21-bit fields of one integer
-  // (a block holds far fewer than 2^21 points)
-  double dsum = (double)ps.defect, mx = (double)ps.maxd;
-  unsigned long long cnt = (unsigned long long)ps.flips |
-                           ((unsigned long long)ps.nonfinite << 21) |
-                           ((unsigned long long)ps.fallback << 42);
-  auto warp_fold = [&]() {
+  sh.defect[tid] = ps.defect;
+  unsigned long long mx;
+  if constexpr (sizeof(R) == 4) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(ps.maxd));
+    mx = (unsigned long long)__double_as_longlong((double)__uint_as_float(m));
+  } else {
+    mx = warp_max_u64((unsigned long long)__double_as_longlong(ps.maxd));
+  }
+  const unsigned fl = __reduce_add_sync(0xffffffffu, (unsigned)ps.flips);
+  unsigned fb = 0, nf = 0;
+  if (__any_sync(0xffffffffu, ps.fallback | ps.nonfinite)) {
+    fb = __reduce_add_sync(0xffffffffu, (unsigned)ps.fallback);
+    nf = __reduce_add_sync(0xffffffffu, (unsigned)ps.nonfinite);
+  }
+  if (l == 0) {
+    sh.maxd[w] = mx;
+    sh.cnt[0][w] = fl;
+    sh.cnt[1][w] = fb;
+    sh.cnt[2][w] = nf;
+  }
+}
+
+// Returns (thread 0) whether this block arrived last; other threads: false.
+template <typename R, int NT>
+__device__ __forceinline__ bool stats_arrive(const StatsPtrs& sp, const StatsShared<R, NT>& sh) {
+  const int tid = threadIdx.x;
+  if (tid >= 32) return false;
+  const int nt = blockDim.x, nw = (nt + 31) >> 5;
+  double d = 0.0;
+  for (int i = tid; i < nt; i += 32) d += (double)sh.defect[i];
+  d = warp_sum(d);
+  const bool in = tid < nw;
+  const unsigned long long mx = warp_max_u64(in ? sh.maxd[tid] : 0ull);
+  const unsigned fl = __reduce_add_sync(0xffffffffu, in ? sh.cnt[0][tid] : 0u);
+  const unsigned fb = __reduce_add_sync(0xffffffffu, in ? sh.cnt[1][tid] : 0u);
+  const unsigned nf = __reduce_add_sync(0xffffffffu, in ? sh.cnt[2][tid] : 0u);
+  if (tid != 0) return false;
+  sp.rb.part[blockIdx.x] = d;
+  sp.rb.rec[blockIdx.x] = BlockRecord{mx, 0ull, fl, fb, nf, 0u};
+  return arrive_acq_rel(&sp.rb.gcount[0]) == gridDim.x - 1;
+}
+
+template <typename R, int NT>
+__device__ __forceinline__ void stats_finish(long long P, double tau, const StatsPtrs& sp, bool last,
+                                             StatsShared<R, NT>& sh) {
+  const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
+  if (tid == 0) sh.last = last ? 1 : 0;
+  __syncthreads();
+  if (!sh.last) return;
+  // thread 0's acquire and the barrier order every block's record before these reads
+  const int nb = (int)gridDim.x, nt = (int)blockDim.x;
+  const int ne = sp.epart ? (int)__ldcg(&sp.st->nep) : 0;
+  double d = 0.0, e = 0.0;
+  unsigned long long mx = 0, fl = 0, fb = 0, nf = 0;
+#pragma unroll 4
+  for (int i = tid; i < nb; i += nt) {
+    d += __ldcg(&sp.rb.part[i]);
+    const BlockRecord* r = &sp.rb.rec[i];
+    const unsigned long long m = __ldcg(&r->maxd_bits);
+    const uint4 c = __ldcg(reinterpret_cast<const uint4*>(&r->flips));
+    mx = m > mx ? m : mx;
+    fl += c.x;
+    fb += c.y;
+    nf += c.z;
+  }
+#pragma unroll 4
+  for (int i = tid; i < ne; i += nt) e += __ldcg(&sp.epart[i]);
+  auto fold = [&]() {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+      d += __shfl_xor_sync(0xffffffffu, d, o);
+      e += __shfl_xor_sync(0xffffffffu, e, o);
+      fl += __shfl_xor_sync(0xffffffffu, fl, o);
+      fb += __shfl_xor_sync(0xffffffffu, fb, o);
+      nf += __shfl_xor_sync(0xffffffffu, nf, o);
     }
+    mx = warp_max_u64(mx);
   };
-  warp_fold();
-  __syncthreads();  // the slots may still be read by an earlier reduction
+  fold();
+  __shared__ unsigned long long tot[3][16];
   if (l == 0) {
-    redd[w] = dsum;
-    redd[16 + w] = mx;
-    redi[w] = (int)(unsigned)cnt;
-    redi[16 + w] = (int)(unsigned)(cnt >> 32);
+    sh.sum[0][w] = d;
+    sh.sum[1][w] = e;
+    sh.maxd[w] = mx;
+    tot[0][w] = fl;
+    tot[1][w] = fb;
+    tot[2][w] = nf;
   }
   __syncthreads();
-  if (w == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    const bool in = l < nw;
-    dsum = in ? redd[l] : 0.0;
-    mx = in ? redd[16 + l] : 0.0;
-    cnt = in ? ((unsigned long long)(unsigned)redi[l] | ((unsigned long long)(unsigned)redi[16 + l] << 32))
-             : 0ull;
-    warp_fold();
+  if (w != 0) return;
+  const bool in = l < ((nt + 31) >> 5);
+  d = in ? sh.sum[0][l] : 0.0;
+  e = in ? sh.sum[1][l] : 0.0;
+  mx = in ? sh.maxd[l] : 0ull;
+  fl = in ? tot[0][l] : 0ull;
+  fb = in ? tot[1][l] : 0ull;
+  nf = in ? tot[2][l] : 0ull;
+  fold();
+  if (tid != 0) return;
+  RunState* st = sp.st;
+  const long long slot = st->step & (kRing - 1);
+  if (sp.epart) {  // deferred energy of this step's input; the defect of A_s is still in st->defect
+    const double Pd = (double)P;
+    const double E_tau = (e / Pd + st->defect) / (Pd * tau);
+    st->energy_last = E_tau;
+    sp.hist.energy[slot] = E_tau;
   }
-  const int fl = (int)(cnt & 0x1FFFFFull);
-  const int nfin = (int)((cnt >> 21) & 0x1FFFFFull);
-  const int nfb = (int)(cnt >> 42);
-  if (tid == 0) {
-    atomicMax(&sp.st->maxdelta_bits, (unsigned long long)__double_as_longlong(mx));
-    if (fl) atomicAdd(&sp.st->flips, (unsigned long long)fl);
-    if (nfin) atomicAdd(&sp.st->nonfinite, (unsigned long long)nfin);
-    if (nfb) atomicAdd(&sp.st->fallback, (unsigned long long)nfb);
-  }
-  double all, esum = 0.0;
-  // deferred energy of this step's input: the multiplier pass's partials
-  // (block order), summed by the last block with the defects; the defect of
-  // A_s is still in st->defect
-  if (grid_sum(dsum, sp.rb, redd, s_flag, &all, sp.epart, sp.epart ? &sp.st->nep : nullptr, &esum)) {
-    if (tid == 0) {
-      RunState* st = sp.st;
-      const long long slot = st->step & (kRing - 1);
-      if (sp.epart) {
-        const double Pd = (double)P;
-        const double E_tau = (esum / Pd + st->defect) / (Pd * tau);
-        st->energy_last = E_tau;
-        sp.hist.energy[slot] = E_tau;
-      }
-      st->defect = all;
-      const double md = __longlong_as_double((long long)atomicAdd(&st->maxdelta_bits, 0ull));
-      const unsigned long long f = atomicAdd(&st->flips, 0ull);
-      const unsigned long long nb = atomicAdd(&st->fallback, 0ull);
-      const unsigned long long nn = atomicAdd(&st->nonfinite, 0ull);
-      sp.hist.maxdelta[slot] = md;
-      sp.hist.flips[slot] = (long long)f;
-      sp.hist.fallback[slot] = (long long)nb;
-      sp.hist.nonfinite[slot] = (long long)nn;
-      if (sp.tol >= 0.0 && f == 0 && md <= sp.tol) st->stop = 1;
-      st->maxdelta_bits = 0;
-      st->flips = 0;
-      st->fallback = 0;
-      st->nonfinite = 0;
-      st->step += 1;
-    }
-  }
+  st->defect = d;
+  const double md = __longlong_as_double((long long)mx);
+  sp.hist.maxdelta[slot] = md;
+  sp.hist.flips[slot] = (long long)fl;
+  sp.hist.fallback[slot] = (long long)fb;
+  sp.hist.nonfinite[slot] = (long long)nf;
+  if (sp.tol >= 0.0 && fl == 0 && md <= sp.tol) st->stop = 1;
+  st->step += 1;
+  sp.rb.gcount[0] = 0;
 }
 
 template <typename R, int NM, int MODE>
@@ -266,8 +340,8 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
   using V = typename VT<R>::V;
   constexpr int C = NM * NM, Q = (C + 1) / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double redd[32];
-  __shared__ int redi[32];
+  __shared__ double redd[MODE == ROW_FWD ? 32 : 1];
+  __shared__ StatsShared<R, MODE == ROW_INV_PROJECT_FWD ? kMaxThreads : 1> sh;
   __shared__ int s_flag, s_nfb;
   if (sp.respect_stop && *(volatile int*)&sp.st->stop) return;
 
@@ -276,7 +350,7 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
   const int S = row_pad(nx);
   const RowLayout lay{S};
   const long long P = g.P;
-  const long long off = (long long)blockIdx.x * nx;
+  long long off = (long long)blockIdx.x * nx;
   const int T = blockDim.x, tid = threadIdx.x;
   const V* tw = static_cast<const V*>(t.tw[0]);
   const bool is_f32 = sizeof(R) == 4;
@@ -307,7 +381,13 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
     return;
   }
 
-  // inverse modes: load the spectrum rows (asynchronous copies)
+  // inverse modes: load the spectrum rows (asynchronous copies).  The
+  // projecting pass walks its rows with a stride of the grid (at most the
+  // blocks that fit on the device), so that a block reduces its statistics once.
+  PointStats<R> ps;
+  bool last = false;
+  const long long gstride = (long long)gridDim.x * nx;
+  for (;; off += gstride) {
 #pragma unroll
   for (int q = 0; q < Q; ++q)
     for (int x = tid; x < nx; x += T) cp_async_elem(&s[lay.addr(q, x)], &W[q * P + off + x]);
@@ -332,7 +412,6 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
   int* fbX = reinterpret_cast<int*>(fbM + kFallbackCap * C);
   if (tid == 0) s_nfb = 0;
   __syncthreads();
-  PointStats<R> ps;
   for (int x = tid; x < nx; x += T) {
     R old[C];
 #pragma unroll
@@ -379,15 +458,22 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
       finish_point<NM>(A, P, off, x, old, b, sg, s + lay.addr(0, x), lay.S, ps);
     }
   }
+  const bool end = off + gstride >= P;
+  if (MODE == ROW_INV_PROJECT_FWD && end && sp.do_stats) stats_park(ps, sh);
   __syncthreads();
+  if (MODE == ROW_INV_PROJECT_FWD && end && sp.do_stats) last = stats_arrive(sp, sh);
   fft_fwd(s, lay, nx, Q, t.plan[0], tw);
 #pragma unroll
   for (int q = 0; q < Q; ++q)
     for (int x = tid; x < nx; x += T) W[q * P + off + x] = s[lay.addr(q, x)];
+  if (end) break;
+  __syncthreads();  // the row is in W: its slots are free
+  }
 
-  if (!sp.do_stats) return;
-  finalize_step_stats(g.P, g.tau, sp, ps, redd, redi, &s_flag);
+  if (MODE != ROW_INV_PROJECT_FWD || !sp.do_stats) return;
+  stats_finish(g.P, g.tau, sp, last, sh);
 }
+
 
 // Strided-axis pass (y in 2-D; y and z in 3-D).  One block owns a tile of tx
 // adjacent x-columns of one complex plane along the whole axis.
@@ -532,19 +618,64 @@ __device__ __forceinline__ R class_pair_checked(const R* m, R* tp, R* tm, R& dE,
   return smin;
 }
 
-// keys[x] = desc_key(dE(x)) for the diffused field At.
-template <typename R, int NM>
-__global__ void __launch_bounds__(256)
-k_vp_delta(long long P, const R* __restrict__ At, unsigned long long* keys, R fb) {
+template <int NM, typename R> __device__ __forceinline__ R det_value(const R* m) {
+  if constexpr (NM == 1) return m[0];
+  else if constexpr (NM == 2) return m[0] * m[3] - m[1] * m[2];
+  else
+    return m[0] * (m[4] * m[8] - m[5] * m[7]) - m[1] * (m[3] * m[8] - m[5] * m[6]) +
+           m[2] * (m[3] * m[7] - m[4] * m[6]);
+}
+
+// keys[x] = desc_key(dE(x)) for the diffused field At.  SELECT: the same pass
+// counts the points of A with det A(x) > 0 (where n_plus < 0 asks for that
+// number) and runs the first pass of the selection, so that neither reads a
+// field again.
+template <typename R, int NM, bool SELECT>
+__global__ void __launch_bounds__(kSelThreads)
+k_vp_delta(long long P, const R* __restrict__ At, const R* __restrict__ A, unsigned long long* keys, R fb,
+           SelectState* ss, long long n_plus) {
   constexpr int C = NM * NM;
+  __shared__ unsigned int h[SELECT ? kSelBins : 1];
+  __shared__ unsigned int part[kSelThreads / 32];
+  __shared__ int s_flag;
+  if constexpr (SELECT) sel_clear(h);
+  int pos = 0;
   for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < P;
        x += (long long)gridDim.x * blockDim.x) {
     R m[C], tp[C], tm[C], dE;
     int fbk = 0;
 #pragma unroll
     for (int c = 0; c < C; ++c) m[c] = At[c * P + x];
+    if (SELECT && n_plus < 0) {
+      R o[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) o[c] = A[c * P + x];
+      pos += det_value<NM>(o) > R(0) ? 1 : 0;
+    }
     class_pair_checked<NM>(m, tp, tm, dE, fb, fbk);
-    keys[x] = desc_key((double)dE);
+    const unsigned long long key = desc_key((double)dE);
+    keys[x] = key;
+    if constexpr (SELECT) atomicAdd(&h[(unsigned)(key >> 53)], 1u);
+  }
+  if constexpr (SELECT) {
+    if (n_plus < 0) {
+      const unsigned w = __reduce_add_sync(0xffffffffu, (unsigned)pos);
+      if ((threadIdx.x & 31) == 0 && w) atomicAdd(&ss->positive, (unsigned long long)w);
+    }
+    if (!sel_flush(h, ss, &s_flag)) return;
+    const unsigned long long n =
+        n_plus < 0 ? *reinterpret_cast<volatile unsigned long long*>(&ss->positive) : (unsigned long long)n_plus;
+    int digit = 0;
+    unsigned long long rest = 0;
+    bool whole = false;
+    const bool mine = sel_pick(ss, n, part, digit, rest, whole);
+    if (mine) sel_record_key(ss, 0ull, 0, digit, rest, whole);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      ss->n_plus = n;
+      ss->positive = 0;
+      if (n == 0) ss->done = 1;  // no bucket holds rank 0: nothing is selected
+    }
   }
 }
 
@@ -560,13 +691,7 @@ k_count_positive(long long P, const R* __restrict__ A, unsigned long long* count
     R m[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) m[c] = A[c * P + x];
-    R d;
-    if constexpr (NM == 1) d = m[0];
-    else if constexpr (NM == 2) d = m[0] * m[3] - m[1] * m[2];
-    else
-      d = m[0] * (m[4] * m[8] - m[5] * m[7]) - m[1] * (m[3] * m[8] - m[5] * m[6]) +
-          m[2] * (m[3] * m[7] - m[4] * m[6]);
-    cnt += (d > R(0)) ? 1 : 0;
+    cnt += (det_value<NM>(m) > R(0)) ? 1 : 0;
   }
   cnt = block_sum(cnt, redi);
   if (threadIdx.x == 0 && cnt) atomicAdd(count, (unsigned long long)cnt);
@@ -579,9 +704,7 @@ __global__ void __launch_bounds__(256)
 k_vp_assign(long long P, const R* __restrict__ At, R* A, const unsigned long long* __restrict__ keys,
             const SelectState* __restrict__ ss, StatsPtrs sp, R fb) {
   constexpr int C = NM * NM;
-  __shared__ double redd[32];
-  __shared__ int redi[32];
-  __shared__ int s_flag;
+  __shared__ StatsShared<R, 256> sh;
   if (sp.respect_stop && *(volatile int*)&sp.st->stop) return;
   const unsigned long long n_plus = ss->n_plus;
   const unsigned long long kh = ss->hi;
@@ -614,27 +737,29 @@ k_vp_assign(long long P, const R* __restrict__ At, R* A, const unsigned long lon
     }
     ps.maxd = fmax(ps.maxd, d);
     ps.defect += R(NM) - nb;
-    R od;
-    if constexpr (NM == 1) od = old[0];
-    else if constexpr (NM == 2) od = old[0] * old[3] - old[1] * old[2];
-    else
-      od = old[0] * (old[4] * old[8] - old[5] * old[7]) - old[1] * (old[3] * old[8] - old[5] * old[6]) +
-           old[2] * (old[3] * old[7] - old[4] * old[6]);
+    const R od = det_value<NM>(old);
     ps.flips += ((od > R(0)) != sel) ? 1 : 0;
   }
   if (!sp.do_stats) return;
-  finalize_step_stats(P, 0.0, sp, ps, redd, redi, &s_flag);  // the energy is the FGI pass's (no epart)
+  stats_park(ps, sh);
+  __syncthreads();
+  const bool last = stats_arrive(sp, sh);
+  stats_finish(P, 0.0, sp, last, sh);  // the energy is the FGI pass's (no epart)
 }
 
 template <typename R>
-cudaError_t launch_volume(int which, const Geom& g, const R* At, R* A, unsigned long long* keys,
+cudaError_t launch_volume(VolumePass which, const Geom& g, const R* At, R* A, unsigned long long* keys,
                           SelectState* ss, const StatsPtrs& sp, double fb, int blocks,
-                          cudaStream_t s) {
+                          cudaStream_t s, long long n_plus) {
   const R f = (R)fb;
 #define MBO_VP_CASE(NM)                                                                         \
   if (g.n == NM) {                                                                              \
-    if (which == 0) k_vp_delta<R, NM><<<blocks, 256, 0, s>>>(g.P, At, keys, f);                 \
-    else if (which == 1) k_count_positive<R, NM><<<blocks, 256, 0, s>>>(g.P, A, &ss->n_plus);   \
+    if (which == VP_DELTA)                                                                      \
+      k_vp_delta<R, NM, false><<<blocks, kSelThreads, 0, s>>>(g.P, At, A, keys, f, ss, 0);      \
+    else if (which == VP_DELTA_SELECT)                                                          \
+      k_vp_delta<R, NM, true><<<blocks, kSelThreads, 0, s>>>(g.P, At, A, keys, f, ss, n_plus);  \
+    else if (which == VP_COUNT)                                                                 \
+      k_count_positive<R, NM><<<blocks, 256, 0, s>>>(g.P, A, &ss->n_plus);                      \
     else k_vp_assign<R, NM><<<blocks, 256, 0, s>>>(g.P, At, A, keys, ss, sp, f);                \
     return cudaGetLastError();                                                                  \
   }
@@ -658,6 +783,25 @@ template <typename K> static cudaError_t set_smem(K kernel, size_t bytes, size_t
   return e;
 }
 
+// Blocks of a kernel that fit on the current device at once (at least one per
+// SM).  `last` keeps the last answer with its question (threads, shared bytes,
+// device) in one word, so that a loop of steps asks the runtime once.
+template <typename K>
+static int resident_blocks(K kernel, int threads, size_t smem, std::atomic<unsigned long long>& last) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const unsigned long long key = ((unsigned long long)(dev & 63) << 30 | (unsigned long long)threads << 20 |
+                                  (unsigned long long)(smem >> 4 & 0xFFFFF)) << 20;
+  const unsigned long long was = last.load(std::memory_order_relaxed);
+  if ((was & ~0xFFFFFull) == key && (was & 0xFFFFF)) return (int)(was & 0xFFFFF);
+  int sms = 1, per_sm = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+  const int n = sms * (per_sm > 0 ? per_sm : 1);
+  last.store(key | (unsigned long long)n, std::memory_order_relaxed);
+  return n;
+}
+
 template <typename R, int NM, int MODE>
 static cudaError_t launch_row_nm(const Geom& g, const Tables<R>& t, const R* Ain, R* A, void* W,
                                  const StatsPtrs& sp, R fb, int threads, cudaStream_t s,
@@ -667,7 +811,11 @@ static cudaError_t launch_row_nm(const Geom& g, const Tables<R>& t, const R* Ain
   const size_t smem = row_smem_bytes(g, sizeof(R), MODE == ROW_INV_PROJECT_FWD);
   cudaError_t e = set_smem(k, smem, done);
   if (e != cudaSuccess || prepare_only) return e;
-  const int rows = g.nz * g.ny;
+  int rows = g.nz * g.ny;
+  if (MODE == ROW_INV_PROJECT_FWD) {
+    static std::atomic<unsigned long long> fits{0};
+    rows = std::min(rows, resident_blocks(k, threads, smem, fits));
+  }
   k<<<rows, threads, smem, s>>>(g, t, Ain, A, static_cast<typename VT<R>::V*>(W), sp, fb);
   return cudaGetLastError();
 }
@@ -801,8 +949,8 @@ template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>
                                       const CUtensorMap*, int, const void*, long long);        \
   template cudaError_t launch_project<R>(const Geom&, const R*, R*, int8_t*, double,          \
                                          cudaStream_t);                                        \
-  template cudaError_t launch_volume<R>(int, const Geom&, const R*, R*, unsigned long long*,   \
+  template cudaError_t launch_volume<R>(VolumePass, const Geom&, const R*, R*, unsigned long long*, \
                                         SelectState*, const StatsPtrs&, double, int,           \
-                                        cudaStream_t);
+                                        cudaStream_t, long long);
 
 }  // namespace mbo

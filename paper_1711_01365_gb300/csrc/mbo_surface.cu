@@ -1303,14 +1303,14 @@ mbo_status mbo_surface_step_volume(mbo_surface s, void* A, double volume, mbo_st
   g.C = s->C;
   const StatsPtrs none{};
   const int blocks = (int)std::min<long long>((s->nq + 255) / 256, 152 * 16);
-  auto vol = [&](int which) {
+  auto vol = [&](VolumePass which) {
     return s->dtype == MBO_F32
                ? launch_volume<float>(which, g, static_cast<const float*>(s->Au), static_cast<float*>(A),
                                       s->vkeys, s->vss, none, 0.0, blocks, st)
                : launch_volume<double>(which, g, static_cast<const double*>(s->Au), static_cast<double*>(A),
                                        s->vkeys, s->vss, none, 0.0, blocks, st);
   };
-  SCK(vol(0));
+  SCK(vol(VP_DELTA));
   if (volume < 0) {
     SCK(cudaMemsetAsync(&s->vws->target, 0, sizeof(unsigned long long), st));
 #define MBO_WVOL(T, NM)                                                                              \
@@ -1331,7 +1331,7 @@ mbo_status mbo_surface_step_volume(mbo_surface s, void* A, double volume, mbo_st
     k_wselect_pick<<<1, 32, 0, st>>>(s->vws, s->vss, d);
   }
   SCK(cudaGetLastError());
-  SCK(vol(2));
+  SCK(vol(VP_ASSIGN));
   SCK(cudaMemsetAsync(s->st, 0, sizeof(SurfStats), st));
   const unsigned pb = (unsigned)((s->nq + kProjThreads - 1) / kProjThreads);
 #define MBO_SDELTA(T, NM)                                                                   \

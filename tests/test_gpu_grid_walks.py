@@ -1,0 +1,79 @@
+"""Passes that walk their work with a stride of the grid, and the selection of
+the volume-preserving step, at the sizes where such loops can go wrong.
+
+* A projecting x pass over more rows than blocks fit on the GPU (72^2 x 96, and
+  4096 two-row groups of 256 points): the step's statistics against the fields
+  it read and wrote, its field against the unfused calls.
+* The radix selection for n = 1, where dE = 2 A~ and the chosen set is known
+  exactly from the diffused field: ties over the whole grid, ties across the
+  threshold, every n_plus at the ends of the range and of the 11-bit digits.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def M():
+    from paper_1711_01365_gb300 import build
+    build.build()
+    from paper_1711_01365_gb300 import mbo
+    return mbo
+
+
+@pytest.mark.parametrize("dims,dtype", [((72, 72, 96), "f32"), ((72, 72, 96), "f64"), ((64, 128, 256), "f32"),
+                                        ((3, 81), "f64"), ((2, 2), "f32")])
+def test_step_statistics_over_many_rows(M, dims, dtype):
+    n, tau = 2, 3.0 / max(dims) ** 2
+    t = torch.float32 if dtype == "f32" else torch.float64
+    g = torch.Generator(device="cuda").manual_seed(5)
+    raw = torch.randn((n * n,) + dims, generator=g, device="cuda", dtype=torch.float64).to(t)
+    h = M.Mbo(dims, n, tau, dtype)
+    A = torch.empty_like(raw)
+    h.project(raw, A)
+    old = A.clone()
+    At, B = torch.empty_like(A), torch.empty_like(A)
+    h.diffuse(old, At)
+    h.project(At, B)
+    E = h.lyapunov(old)
+    rec = h.step(A, want_stats=True)
+    assert rec["max_delta"] == float((A - old).abs().max())
+    det = lambda F: F[0] * F[3] - F[1] * F[2]  # noqa: E731
+    assert rec["det_flips"] == int(((det(A) >= 0) != (det(old) >= 0)).sum())
+    assert rec["energy"] == pytest.approx(E, rel=1e-6 if dtype == "f32" else 1e-12)
+    # the fused and the unfused step differ by rounding where the class is clear
+    far = (At.double()[0] + At.double()[3]).hypot(At.double()[2] - At.double()[1]) - \
+          (At.double()[0] - At.double()[3]).hypot(At.double()[1] + At.double()[2])
+    clear = far.abs() > 1e-2
+    assert float((A - B).abs().amax(0)[clear].max()) <= (2e-5 if dtype == "f32" else 1e-12)
+    h.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("dims", [(2, 2), (32, 64), (48, 54), (128, 192)])
+@pytest.mark.parametrize("kind", ["constant", "two", "random", "tiny"])
+def test_selection_takes_the_largest_lowest_index_first(M, dims, kind, dtype):
+    P = int(np.prod(dims))
+    r = np.random.default_rng(9)
+    F = {"constant": lambda: np.full(dims, 0.25),
+         "two": lambda: np.where(np.arange(P).reshape(dims) % dims[1] < dims[1] // 2, 0.5, -0.75),
+         "random": lambda: r.standard_normal(dims),
+         "tiny": lambda: 1e-30 * r.standard_normal(dims)}[kind]()
+    t = torch.float32 if dtype == "f32" else torch.float64
+    h = M.Mbo(dims, 1, 4.0 / min(dims) ** 2, dtype)
+    A0 = torch.tensor(F, dtype=t, device="cuda")[None].contiguous()
+    At = torch.empty_like(A0)
+    h.diffuse(A0, At)
+    order = np.argsort(-At.cpu().numpy().ravel(), kind="stable")
+    for n_plus in sorted({0, 1, P // 3, min(2047, P), min(2048, P), P - 1, P}):
+        A = A0.clone()
+        h.step_volume(A, n_plus)
+        want = -np.ones(P)
+        want[order[:n_plus]] = 1.0
+        assert np.array_equal(A.cpu().numpy().ravel(), want), n_plus
+    A = A0.clone()  # the volume of the field itself
+    h.step_volume(A, -1)
+    assert int((A > 0).sum()) == int((A0 > 0).sum())
+    h.close()
