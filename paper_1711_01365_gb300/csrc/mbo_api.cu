@@ -52,21 +52,48 @@ FastDiv make_div(unsigned d) {
   return f;
 }
 
-// Radix plan: the power of two in ceil(a/4) stages of 16 / 8 / 4 / 2 (bits
-// spread evenly, larger radices first), then one radix-3 stage per factor 3.
-// Stage twiddle offsets are assigned in stage order.
+// Radix plan of N = 2^a 3^b: as few stages of radix 16, 12, 9, 8, 6, 4, 3 or 2
+// as possible, and among those plans the one of least butterfly work (operations
+// per point of a length-r DFT, by how the registers compute it).  The stages
+// with the most factors of two come first, so that the spans below them stay
+// multiples of 8 (affine addressing) as long as possible.  Stage twiddle
+// offsets are assigned in stage order.
+struct RadixCost { int r, a, b; double ops; };
+const RadixCost kRadix[] = {{16, 4, 0, 10.5}, {12, 2, 1, 9.3}, {9, 0, 2, 10.2}, {8, 3, 0, 7.0},
+                            {6, 1, 1, 7.3},   {4, 2, 0, 4.0},  {3, 0, 1, 5.3},  {2, 1, 0, 2.0}};
+
+void search_plan(int a, int b, int from, int depth, int* cur, double ops, int& best_n, double& best_ops,
+                 int* best) {
+  if (a == 0 && b == 0) {
+    if (depth < best_n || (depth == best_n && ops < best_ops)) {
+      best_n = depth;
+      best_ops = ops;
+      std::copy(cur, cur + depth, best);
+    }
+    return;
+  }
+  if (depth >= best_n || depth >= kMaxStages) return;
+  for (int i = from; i < 8; ++i) {
+    const RadixCost& r = kRadix[i];
+    if (r.a > a || r.b > b) continue;
+    cur[depth] = r.r;
+    search_plan(a - r.a, b - r.b, i, depth + 1, cur, ops + r.ops, best_n, best_ops, best);
+  }
+}
+
 Plan make_plan(int N) {
   Plan p{};
   p.len = N;
   int a, b;
   factor23(N, a, b);
-  int rad[kMaxStages];
-  int ns = 0;
-  if (a > 0) {
-    const int n2 = (a + 3) / 4;
-    for (int i = 0; i < n2; ++i) rad[ns++] = 1 << (a / n2 + (i < a % n2 ? 1 : 0));
-  }
-  for (int i = 0; i < b; ++i) rad[ns++] = 3;
+  int rad[kMaxStages], cur[kMaxStages];
+  int ns = kMaxStages + 1;
+  double ops = 0.0;
+  search_plan(a, b, 0, 0, cur, 0.0, ns, ops, rad);
+  std::stable_sort(rad, rad + ns, [](int x, int y) {
+    auto twos = [](int v) { int t = 0; while (v % 2 == 0) { v /= 2; ++t; } return t; };
+    return twos(x) > twos(y);
+  });
   p.nst = ns;
   int lb = N, tw = 0;
   for (int i = 0; i < ns; ++i) {
@@ -131,6 +158,12 @@ void digit_positions(const Plan& p, int N, std::vector<int>& pos) {
 int pick_tx(int nx, int cap) {
   int t = 1;
   while (t < cap && nx % (2 * t) == 0) t *= 2;
+  return t;
+}
+
+int net_tile(int nx, int cap) {
+  int t = 1;
+  while (t < cap && t < nx) t *= 2;
   return t;
 }
 
@@ -383,17 +416,21 @@ cudaError_t row_launch(mbo_ctx* h, RowMode mode, const void* Ain, void* Aout, co
 // its step statistics) into L2 while it transforms.
 constexpr size_t kL2HintBytes = 96u << 20;
 
+int net_width(const mbo_ctx* h, int tx);
+
 cudaError_t axis_launch(mbo_ctx* h, AxisMode mode, int axis, const StatsPtrs& sp, cudaStream_t s,
                         const void* l2_hint) {
+  const bool warp = h->dtype == MBO_F32 && h->tf.plan[axis].lq;
+  const int tx = warp ? h->tx : net_width(h, h->tx);
   const size_t abytes = (size_t)h->g.C * (size_t)h->g.P * h->elem;
   const size_t wbytes = (size_t)h->g.Q * (size_t)h->g.P * 2 * h->elem;
   if (abytes + wbytes > kL2HintBytes) l2_hint = nullptr;
   pdl_flag() = h->pdl;
   if (h->dtype == MBO_F32)
-    return launch_axis<float>(mode, axis, h->g, h->tf, h->W, sp, h->tx, h->axis_threads, s,
+    return launch_axis<float>(mode, axis, h->g, h->tf, h->W, sp, tx, h->axis_threads, s,
                               h->wmap_ok[axis] ? &h->wmap[axis] : nullptr, h->axis_stages,
                               l2_hint, l2_hint ? (long long)abytes : 0);
-  return launch_axis<double>(mode, axis, h->g, h->td, h->W, sp, h->tx, h->axis_threads, s);
+  return launch_axis<double>(mode, axis, h->g, h->td, h->W, sp, tx, h->axis_threads, s);
 }
 
 // Transform passes between the forward and the inverse x pass.
@@ -463,6 +500,15 @@ template <typename R> __global__ void k_tune_fill(R* A, long long n) {
   }
 }
 
+// Columns per tile of the handle's network strided passes where the tile width
+// setting is tx: an explicit width as it is; else a narrow one, which only the
+// field's width forces (tx divides nx), gives way to a full tile with a ragged
+// last one (64 bytes of each row instead of 16 for nx = 486, 8 for nx = 243).
+int net_width(const mbo_ctx* h, int tx) {
+  const int cap = h->dtype == MBO_F32 ? 8 : 4;
+  return h->cfg.axis_tx || tx >= cap ? tx : net_tile(h->g.nx, cap);
+}
+
 bool shape_fits(mbo_ctx* h, const LaunchShape& c, int maxsm) {
   const Geom& g = h->g;
   if (c.tx < 1 || g.nx % c.tx) return false;
@@ -471,7 +517,7 @@ bool shape_fits(mbo_ctx* h, const LaunchShape& c, int maxsm) {
     if (h->dtype == MBO_F32 && h->tf.plan[ax].lq) {
       const int wt = warp_tile(L, g.nx, c.tx);
       if (!wt || wcol_smem_bytes(L, wt, c.stages) > (size_t)maxsm) return false;
-    } else if (axis_smem_bytes(L, c.tx, h->elem) > (size_t)maxsm) {
+    } else if (axis_smem_bytes(L, net_width(h, c.tx), h->elem) > (size_t)maxsm) {
       return false;
     }
   }
@@ -487,8 +533,8 @@ cudaError_t apply_shape(mbo_ctx* h, const LaunchShape& c) {
   h->xpers = c.xpers;
   invalidate_graph(h);
   const Geom& g = h->g;
-  cudaError_t e = h->dtype == MBO_F32 ? prepare_kernels<float>(g, h->tf, h->tx, h->axis_stages)
-                                      : prepare_kernels<double>(g, h->td, h->tx, 1);
+  cudaError_t e = h->dtype == MBO_F32 ? prepare_kernels<float>(g, h->tf, h->tx, net_width(h, h->tx), h->axis_stages)
+                                      : prepare_kernels<double>(g, h->td, h->tx, net_width(h, h->tx), 1);
   if (e != cudaSuccess) return e;
   if (h->dtype == MBO_F32) {
     for (int ax = 1; ax < g.ndim; ++ax) {
@@ -782,7 +828,7 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
       as = std::max(as, wcol_smem_bytes(L, wt, h->axis_stages));
       min_tx = std::min(min_tx, wt);
     } else {
-      as = std::max(as, axis_smem_bytes(L, h->tx, h->elem));
+      as = std::max(as, axis_smem_bytes(L, net_width(h, h->tx), h->elem));
     }
   }
   int maxsm = 0;
@@ -851,8 +897,8 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
     cudaMemcpy(h->tabs, tb.bytes.data(), tb.bytes.size(), cudaMemcpyHostToDevice);
     bind_tables(h, tb, h->td);
   }
-  const cudaError_t pe = dtype == MBO_F32 ? prepare_kernels<float>(g, h->tf, h->tx, h->axis_stages)
-                                          : prepare_kernels<double>(g, h->td, h->tx, 1);
+  const cudaError_t pe = dtype == MBO_F32 ? prepare_kernels<float>(g, h->tf, h->tx, net_width(h, h->tx), h->axis_stages)
+                                          : prepare_kernels<double>(g, h->td, h->tx, net_width(h, h->tx), 1);
   if (pe != cudaSuccess) {
     (void)cudaGetLastError();  // the failed attribute call must not surface at a later launch
     mbo_destroy(h);

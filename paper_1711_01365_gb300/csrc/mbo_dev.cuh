@@ -121,10 +121,67 @@ template <int DIR, typename V> __device__ __forceinline__ void dft16(V* v) {
   }
 }
 
+// Length N1 * N2 with coprime factors (Good 1958): the index maps
+//   n = N2 n1 + N1 n2 mod N,   k = N2 e2 k1 + N1 e1 k2 mod N
+// (e2 N2 = 1 mod N1, e1 N1 = 1 mod N2) leave length-N1 and length-N2 DFTs and
+// no twiddles between them.
+template <int DIR, int N1, int N2, typename V> __device__ __forceinline__ void dft_coprime(V* v) {
+  constexpr int N = N1 * N2;
+  constexpr int e2 = N2 % N1 == 1 ? 1 : N1 - 1, e1 = N1 % N2 == 1 ? 1 : N2 - 1;  // factors 2, 3 and 4
+  static_assert((e2 * N2) % N1 == 1 && (e1 * N1) % N2 == 1, "inverses");
+  V u[N1][N2];
+#pragma unroll
+  for (int n2 = 0; n2 < N2; ++n2) {
+    V a[N1];
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) a[n1] = v[(N2 * n1 + N1 * n2) % N];
+    if constexpr (N1 == 2) dft2<DIR>(a);
+    else dft4<DIR>(a);
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) u[k1][n2] = a[k1];
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < N1; ++k1) {
+    dft3<DIR>(u[k1]);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) v[(N2 * e2 * k1 + N1 * e1 * k2) % N] = u[k1][k2];
+  }
+}
+
+// Length 9 = 3 x 3: n = n2 + 3 n1, k = k1 + 3 k2, twiddles W9^(n2 k1) between.
+template <int DIR, typename V> __device__ __forceinline__ void dft9(V* v) {
+  using R = decltype(v[0].x);
+  const R D = R(DIR);
+  const V w1 = V{R(0.76604444311897803520), D * R(0.64278760968653932632)};   // W9
+  const V w2 = V{R(0.17364817766693034885), D * R(0.98480775301220805937)};   // W9^2
+  const V w4 = V{R(-0.93969262078590838405), D * R(0.34202014332566873304)};  // W9^4
+  V u[3][3];
+#pragma unroll
+  for (int n2 = 0; n2 < 3; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < 3; ++n1) u[n2][n1] = v[n2 + 3 * n1];
+    dft3<DIR>(u[n2]);
+  }
+  u[1][1] = cmul(u[1][1], w1);
+  u[1][2] = cmul(u[1][2], w2);
+  u[2][1] = cmul(u[2][1], w2);
+  u[2][2] = cmul(u[2][2], w4);
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    V a[3] = {u[0][k1], u[1][k1], u[2][k1]};
+    dft3<DIR>(a);
+#pragma unroll
+    for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = a[k2];
+  }
+}
+
 template <int DIR, int RAD, typename V> __device__ __forceinline__ void dft(V* v) {
   if constexpr (RAD == 2) dft2<DIR>(v);
   else if constexpr (RAD == 3) dft3<DIR>(v);
   else if constexpr (RAD == 4) dft4<DIR>(v);
+  else if constexpr (RAD == 6) dft_coprime<DIR, 2, 3>(v);
+  else if constexpr (RAD == 9) dft9<DIR>(v);
+  else if constexpr (RAD == 12) dft_coprime<DIR, 4, 3>(v);
   else if constexpr (RAD == 8) dft8<DIR>(v);
   else dft16<DIR>(v);
 }
@@ -187,6 +244,9 @@ struct ColLayout {
 // butterfly reads and writes the same RAD slots, so threads never hold more
 // than one butterfly and a stage needs only a barrier after it.  Multiplier
 // tables are permuted on the host to the digit-reversed positions.
+//
+// Radices 16, 12, 9, 8, 6, 4, 3 and 2; the plan takes as few stages as they
+// allow (each stage is a round trip through shared memory and a barrier).
 //
 // Stage st works on blocks of length lb = N / (r_0 ... r_{st-1}); a butterfly
 // (block b, offset n1 < m = lb / RAD) owns positions b*lb + n1 + m*j.  Its
@@ -253,6 +313,9 @@ __device__ __forceinline__ void run_stage(V* s, const L& lay, int N, int M, cons
                                           const V* __restrict__ tw) {
   switch (sd.rad) {
     case 16: radix_stage<DIR, 16>(s, lay, N, M, sd, tw); break;
+    case 12: radix_stage<DIR, 12>(s, lay, N, M, sd, tw); break;
+    case 9: radix_stage<DIR, 9>(s, lay, N, M, sd, tw); break;
+    case 6: radix_stage<DIR, 6>(s, lay, N, M, sd, tw); break;
     case 8: radix_stage<DIR, 8>(s, lay, N, M, sd, tw); break;
     case 4: radix_stage<DIR, 4>(s, lay, N, M, sd, tw); break;
     case 3: radix_stage<DIR, 3>(s, lay, N, M, sd, tw); break;

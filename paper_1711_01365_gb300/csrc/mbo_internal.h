@@ -89,14 +89,16 @@ struct Geom {
   int xh;
 };
 
-// Tile count of a strided pass (tiles of tx x-columns, nouter outer rows per plane).
+// Tile count of a strided pass (tiles of tx x-columns, nouter outer rows per
+// plane; the last tile of a row of tiles is ragged where tx does not divide nx,
+// which only the network passes allow).
 __host__ __device__ inline int col_tiles(const Geom& g, int nouter, int tx) {
-  return (g.Q - 1) * nouter * (g.nx / tx) + nouter * (g.xh / tx);
+  return (g.Q - 1) * nouter * ((g.nx + tx - 1) / tx) + nouter * ((g.xh + tx - 1) / tx);
 }
 // Plane q, outer index o and first column x0 of strided-pass tile b.
 __host__ __device__ inline void col_tile(const Geom& g, int nouter, int tx, int b, int& q, int& o,
                                          int& x0) {
-  const int xt = g.nx / tx;
+  const int xt = (g.nx + tx - 1) / tx;
   const int full = (g.Q - 1) * nouter * xt;
   if (b < full) {
     q = b / (nouter * xt);
@@ -104,7 +106,7 @@ __host__ __device__ inline void col_tile(const Geom& g, int nouter, int tx, int 
     o = rem / xt;
     x0 = (rem - o * xt) * tx;
   } else {
-    const int xtl = g.xh / tx;
+    const int xtl = (g.xh + tx - 1) / tx;
     const int rem = b - full;
     q = g.Q - 1;
     o = rem / xtl;
@@ -217,6 +219,9 @@ Plan make_plan(int N);
 Plan axis_plan(const Geom& g, int axis, bool f32);
 int plan_twiddles(const Plan& p);
 int pick_tx(int nx, int cap);
+// Columns per tile of the network strided passes: `cap` (64 bytes a tile row),
+// or the power of two that covers a narrower field.
+int net_tile(int nx, int cap);
 
 // FP32 passes over warp-plan axes (k_warp.cu).
 bool& pdl_flag();  // programmatic dependent launch of these passes (per host thread)
@@ -239,7 +244,7 @@ cudaError_t launch_wcol(AxisMode mode, int axis, const Geom& g, const Tables<flo
 bool wcol_tensor_map(CUtensorMap* map, void* W, const Geom& g, int axis, int tx);
 
 template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>& t, int tx,
-                                                  int stages);
+                                                  int net_tx, int stages);
 template <typename R>
 cudaError_t launch_volume(VolumePass which, const Geom& g, const R* At, R* A, unsigned long long* keys,
                           SelectState* ss, const StatsPtrs& sp, double fb, int blocks,

@@ -504,7 +504,10 @@ k_axis(Geom g, Tables<R> t, typename VT<R>::V* W, StatsPtrs sp, int axis, int lt
   const int mcol = tid & (tx - 1);
   const int p0 = tid >> ltx, dp = T >> ltx;
   const long long gstep = (long long)dp * es;
-  {
+  // the last tile of a row may reach past the field: its columns there hold
+  // nothing, are transformed with the rest and are not stored
+  const bool live = x0 + mcol < g.nx;
+  if (live) {
     const V* src = base + mcol + (long long)p0 * es;
     for (int p = p0; p < L; p += dp, src += gstep) cp_async_elem(&s[lay.addr(mcol, p)], src);
   }
@@ -513,6 +516,7 @@ k_axis(Geom g, Tables<R> t, typename VT<R>::V* W, StatsPtrs sp, int axis, int lt
   if (MODE != AXIS_INV) fft_fwd(s, lay, L, tx, t.plan[axis], tw);
   R acc = R(0);
   if (MODE == AXIS_FGI || MODE == AXIS_ENERGY) {
+    if (live) {
     // the last axis applies g(k) = g_x g_y (g_z); in 3-D the y frequency is
     // the outer index o of this tile (the y pass ran before).
     R go = R(1), omo = R(0);
@@ -538,10 +542,11 @@ k_axis(Geom g, Tables<R> t, typename VT<R>::V* W, StatsPtrs sp, int axis, int lt
         s[e] = V{z.x * f, z.y * f};
       }
     }
+    }
     __syncthreads();
   }
   if (MODE == AXIS_FGI || MODE == AXIS_INV) fft_inv(s, lay, L, tx, t.plan[axis], tw);
-  if (MODE != AXIS_ENERGY) {
+  if (MODE != AXIS_ENERGY && live) {
     V* dst = base + mcol + (long long)p0 * es;
     for (int p = p0; p < L; p += dp, dst += gstep) *dst = s[lay.addr(mcol, p)];
   }
@@ -898,7 +903,7 @@ cudaError_t launch_project(const Geom& g, const R* At, R* B, int8_t* det_sign,
 // launching (so that later launches inside stream capture make no attribute
 // call).
 template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>& tabs, int tx,
-                                                  int stages) {
+                                                  int net_tx, int stages) {
   Tables<R> t{};
   StatsPtrs sp{};
   cudaError_t e = cudaSuccess;
@@ -931,17 +936,17 @@ template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>
 #undef MBO_PREP_ROW
   for (int axis = 1; axis <= (g.ndim == 3 ? 2 : 1) && e == cudaSuccess; ++axis) {
     if (sizeof(R) == 4 && tabs.plan[axis].lq) continue;  // the warp-plan pass above takes this axis
-    e = launch_axis_m<R, AXIS_FWD>(g, t, nullptr, sp, axis, tx, 64, 0, true);
-    if (e == cudaSuccess) e = launch_axis_m<R, AXIS_INV>(g, t, nullptr, sp, axis, tx, 64, 0, true);
-    if (e == cudaSuccess) e = launch_axis_m<R, AXIS_FGI>(g, t, nullptr, sp, axis, tx, 64, 0, true);
+    e = launch_axis_m<R, AXIS_FWD>(g, t, nullptr, sp, axis, net_tx, 64, 0, true);
+    if (e == cudaSuccess) e = launch_axis_m<R, AXIS_INV>(g, t, nullptr, sp, axis, net_tx, 64, 0, true);
+    if (e == cudaSuccess) e = launch_axis_m<R, AXIS_FGI>(g, t, nullptr, sp, axis, net_tx, 64, 0, true);
     if (e == cudaSuccess)
-      e = launch_axis_m<R, AXIS_ENERGY>(g, t, nullptr, sp, axis, tx, 64, 0, true);
+      e = launch_axis_m<R, AXIS_ENERGY>(g, t, nullptr, sp, axis, net_tx, 64, 0, true);
   }
   return e;
 }
 
 #define MBO_INSTANTIATE(R)                                                                     \
-  template cudaError_t prepare_kernels<R>(const Geom&, const Tables<R>&, int, int);            \
+  template cudaError_t prepare_kernels<R>(const Geom&, const Tables<R>&, int, int, int);       \
   template cudaError_t launch_row<R>(RowMode, const Geom&, const Tables<R>&, const R*, R*,     \
                                      void*, const StatsPtrs&, double, int, cudaStream_t);      \
   template cudaError_t launch_axis<R>(AxisMode, int, const Geom&, const Tables<R>&, void*,     \

@@ -102,7 +102,7 @@ mbo_status diffuse_noalloc(const Geom& g, const void* A, void* At, cudaStream_t 
     off = align256(off + (size_t)lens[ax] * sizeof(R));
   }
   if (off > (size_t)MBO_NOALLOC_SCRATCH_BYTES) return MBO_ERR_UNSUPPORTED_SIZE;
-  const int tx = pick_tx(g.nx, sizeof(R) == 4 ? 8 : 4);
+  const int tx = net_tile(g.nx, sizeof(R) == 4 ? 8 : 4);
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MBO_ERR_CUDA;
   // The row and strided passes keep whole rows / column tiles in shared

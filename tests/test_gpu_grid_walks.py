@@ -77,3 +77,34 @@ def test_selection_takes_the_largest_lowest_index_first(M, dims, kind, dtype):
     h.step_volume(A, -1)
     assert int((A > 0).sum()) == int((A0 > 0).sum())
     h.close()
+
+
+@pytest.mark.parametrize("dims", [(486, 18), (243, 9), (162, 27), (81, 6), (54, 36), (9, 2), (27, 3),
+                                  (12, 1458), (1944, 6), (4, 9, 81), (18, 27, 12), (648, 54)])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_network_radices_and_ragged_tiles(M, dims, dtype):
+    """Axes with every radix of the network's plans, and rows that end in a ragged column tile: the
+    diffusion with and without a handle, and the energy, against torch in FP64."""
+    n, tau = 2, 3.0 / max(dims) ** 2
+    t = torch.float32 if dtype == "f32" else torch.float64
+    g = torch.Generator(device="cuda").manual_seed(3)
+    A = torch.randn((n * n,) + dims, generator=g, device="cuda", dtype=torch.float64).to(t)
+    e = 0.0
+    for ax, N in enumerate(dims):
+        k = torch.fft.fftfreq(N, 1.0 / N, device="cuda", dtype=torch.float64)
+        e = e - 4 * np.pi ** 2 * tau * (k * k).reshape([-1 if ax == b else 1 for b in range(len(dims))])
+    F = torch.fft.fftn(A.double(), dim=tuple(range(1, len(dims) + 1)))
+    want = torch.fft.ifftn(F * torch.exp(e), dim=tuple(range(1, len(dims) + 1))).real
+    P = float(np.prod(dims))
+    E = float((-torch.expm1(e) * F.abs().square()).sum() / P + (n - A.double().square().sum(0)).sum()) / (P * tau)
+    h = M.Mbo(dims, n, tau, dtype)
+    out = torch.empty_like(A)
+    h.diffuse(A, out)
+    tol = 4e-6 if dtype == "f32" else 1e-13
+    scale = float(want.abs().max())
+    assert float((out.double() - want).abs().max()) <= tol * max(1.0, scale)
+    M.mbo_diffuse_noalloc(dims, n, tau, M.MBO_F32 if dtype == "f32" else M.MBO_F64, A, out)
+    assert float((out.double() - want).abs().max()) <= tol * max(1.0, scale)
+    scaleE = float((F.abs().square().sum() / P + A.double().square().sum())) / (P * tau)
+    assert abs(h.lyapunov(A) - E) <= (1e-5 if dtype == "f32" else 1e-12) * scaleE
+    h.close()
