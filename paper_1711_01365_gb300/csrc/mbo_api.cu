@@ -59,9 +59,11 @@ FastDiv make_div(unsigned d) {
 // multiples of 8 (affine addressing) as long as possible.  Stage twiddle
 // offsets are assigned in stage order.
 struct RadixCost { int r, a, b; double ops; };
+// (small_code: without 16 and 12)
 const RadixCost kRadix[] = {{16, 4, 0, 10.5}, {12, 2, 1, 9.3}, {9, 0, 2, 10.2}, {8, 3, 0, 7.0},
                             {6, 1, 1, 7.3},   {4, 2, 0, 4.0},  {3, 0, 1, 5.3},  {2, 1, 0, 2.0}};
 
+// from: first entry of kRadix to try
 void search_plan(int a, int b, int from, int depth, int* cur, double ops, int& best_n, double& best_ops,
                  int* best) {
   if (a == 0 && b == 0) {
@@ -81,7 +83,7 @@ void search_plan(int a, int b, int from, int depth, int* cur, double ops, int& b
   }
 }
 
-Plan make_plan(int N) {
+Plan make_plan(int N, bool small_code) {
   Plan p{};
   p.len = N;
   int a, b;
@@ -89,7 +91,8 @@ Plan make_plan(int N) {
   int rad[kMaxStages], cur[kMaxStages];
   int ns = kMaxStages + 1;
   double ops = 0.0;
-  search_plan(a, b, 0, 0, cur, 0.0, ns, ops, rad);
+  search_plan(a, b, small_code ? 2 : 0, 0, cur, 0.0, ns, ops, rad);
+  // 2^10 and 2^11 need four radix-8 stages: always within kMaxStages
   std::stable_sort(rad, rad + ns, [](int x, int y) {
     auto twos = [](int v) { int t = 0; while (v % 2 == 0) { v /= 2; ++t; } return t; };
     return twos(x) > twos(y);
@@ -113,6 +116,8 @@ Plan make_plan(int N) {
   return p;
 }
 
+constexpr long long kSmallCode = 1500000;
+
 Plan axis_plan(const Geom& g, int axis, bool f32) {
   const int N = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
   if (f32 && warp_plan_length(N) && (axis == 0 || warp_tile(N, g.nx, 8) != 0) &&
@@ -123,7 +128,12 @@ Plan axis_plan(const Geom& g, int axis, bool f32) {
     p.lq = N / p.rad0 == 1024 ? 32 : 16;
     return p;
   }
-  return make_plan(N);
+  // FP64 (fixed point): the butterflies of radix 16 and 12 are 45 and 30 KB of
+  // instructions, which every SM fetches once per pass at about 4 KB/us (ncu:
+  // warps wait for instructions first of all); up to kSmallCode elements that
+  // costs more than the stage they save (128^2, n = 2: y pass 29 -> 23 us, x pass
+  // 31 -> 23 us)
+  return make_plan(N, !f32 && g.P * g.Q <= kSmallCode);
 }
 
 int plan_twiddles(const Plan& p) {
@@ -263,6 +273,61 @@ template <typename R> struct TabBuild {
   size_t off_tw[3], off_g[3], off_om[3];
 };
 
+// cos and sin of 2 pi e / N in Q60, by octants.  Inside one, (r / N) pi / 4 in
+// Q62 and the Taylor series in Horner form on 128-bit products (term k of 13 is
+// below 2^-62 there); a few units of 2^-62 off at most.  Extended-precision
+// library calls would do too, but are software on Arm and as slow as the rest
+// of a small plan.
+struct UnitCircle {
+  long long N;
+  explicit UnitCircle(int n) : N(n) {}
+  static long long mul62(long long a, long long b) { return (long long)(((__int128)a * b) >> 62); }
+  // octant o = floor(8 e / N), remainder r = 8 e - o N in [0, N): angle (o + r / N) pi / 4
+  void octant(size_t e, int& o, long long& r) const {
+    o = (int)(8 * (long long)e / N);
+    r = 8 * (long long)e - o * N;
+  }
+  long long base(bool sine, long long r) const {  // cos or sin of (r / N) pi / 4
+    const long long one = 1ll << 62;
+    const __int128 quarter_pi = 3622009729038561421ll;  // pi / 4 in Q62
+    const long long a = (long long)((quarter_pi * r + N / 2) / N), a2 = mul62(a, a);
+    long long v = one;
+    for (int k = 13; k >= 1; --k) v = one - mul62(a2, v) / (sine ? 2 * k * (2 * k + 1) : (2 * k - 1) * 2 * k);
+    if (sine) v = mul62(a, v);
+    return (v + 2) >> 2;
+  }
+  long long cos_q60(size_t e) const {
+    int o;
+    long long r;
+    octant(e, o, r);
+    switch (o) {
+      case 0: return base(false, r);
+      case 1: return base(true, N - r);
+      case 2: return -base(true, r);
+      case 3: return -base(false, N - r);
+      case 4: return -base(false, r);
+      case 5: return -base(true, N - r);
+      case 6: return base(true, r);
+      default: return base(false, N - r);
+    }
+  }
+  long long sin_q60(size_t e) const {
+    int o;
+    long long r;
+    octant(e, o, r);
+    switch (o) {
+      case 0: return base(true, r);
+      case 1: return base(false, N - r);
+      case 2: return base(false, r);
+      case 3: return base(true, N - r);
+      case 4: return -base(true, r);
+      case 5: return -base(false, N - r);
+      case 6: return -base(false, r);
+      default: return -base(true, N - r);
+    }
+  }
+};
+
 template <typename R>
 void build_tables(mbo_ctx* h, TabBuild<R>& tb, Tables<R>& t) {
   const int lens[3] = {h->g.nx, h->g.ny, h->g.nz};
@@ -285,6 +350,13 @@ void build_tables(mbo_ctx* h, TabBuild<R>& tb, Tables<R>& t) {
     const int N = lens[ax];
     const Plan& pl = t.plan[ax];
     R* tw = reinterpret_cast<R*>(&tb.bytes[tb.off_tw[ax]]);
+    if (ax > 0 && N == lens[ax - 1] && pl.lq == t.plan[ax - 1].lq) {  // the same plan: the same tables
+      const size_t tn = (size_t)std::max(plan_twiddles(pl), 1) * 2 * sizeof(R), gn = (size_t)N * sizeof(R);
+      std::memcpy(tw, &tb.bytes[tb.off_tw[ax - 1]], tn);
+      std::memcpy(&tb.bytes[tb.off_g[ax]], &tb.bytes[tb.off_g[ax - 1]], gn);
+      std::memcpy(&tb.bytes[tb.off_om[ax]], &tb.bytes[tb.off_om[ax - 1]], gn);
+      continue;
+    }
     if (pl.lq) {
       // N = rad0 * Mw: the length-Mw table [k2][l] = exp(-2 pi i l k2 / Mw), then
       // the pre-stage twiddles exp(-2 pi i r k' / N) at Mw + (r - 1) Mw + k'
@@ -306,6 +378,7 @@ void build_tables(mbo_ctx* h, TabBuild<R>& tb, Tables<R>& t) {
           tw[2 * i + 1] = (R)(-std::sin(ang));
         }
     }
+    const UnitCircle unit(sizeof(R) == 8 ? N : 1);
     for (int st = 0; st < pl.nst; ++st) {
       const Stage& s = pl.st[st];
       if (s.m <= 1) continue;
@@ -314,8 +387,14 @@ void build_tables(mbo_ctx* h, TabBuild<R>& tb, Tables<R>& t) {
           const long long e = ((long long)n1 * j) % s.lb;
           const double ang = 2.0 * pi * (double)e / (double)s.lb;
           const size_t i = (size_t)s.tw + (size_t)(j - 1) * s.m + n1;
-          tw[2 * i] = (R)std::cos(ang);
-          tw[2 * i + 1] = (R)(-std::sin(ang));
+          if constexpr (sizeof(R) == 8) {  // Q60 limbs of the fixed-point transforms
+            const size_t at = (size_t)e * (size_t)(N / s.lb);
+            const FxTw w = fx_tw(unit.cos_q60(at), -unit.sin_q60(at));
+            std::memcpy(tw + 2 * i, &w, sizeof(w));
+          } else {
+            tw[2 * i] = (R)std::cos(ang);
+            tw[2 * i + 1] = (R)(-std::sin(ang));
+          }
         }
     }
     std::vector<int> pos;
@@ -503,10 +582,17 @@ template <typename R> __global__ void k_tune_fill(R* A, long long n) {
 // Columns per tile of the handle's network strided passes where the tile width
 // setting is tx: an explicit width as it is; else a narrow one, which only the
 // field's width forces (tx divides nx), gives way to a full tile with a ragged
-// last one (64 bytes of each row instead of 16 for nx = 486, 8 for nx = 243).
+// last one (64 bytes of each row instead of 16 for nx = 486, 8 for nx = 243), and
+// a field with fewer tiles than SMs takes narrower ones (128^2, n = 2, FP64 y
+// pass: 4 columns 23.0 us, 1 column 19.8 us), down to 16 bytes of a row.
 int net_width(const mbo_ctx* h, int tx) {
-  const int cap = h->dtype == MBO_F32 ? 8 : 4;
-  return h->cfg.axis_tx || tx >= cap ? tx : net_tile(h->g.nx, cap);
+  const bool f32 = h->dtype == MBO_F32;
+  const int cap = f32 ? 8 : 4;
+  if (h->cfg.axis_tx) return tx;
+  int w = tx >= cap ? tx : net_tile(h->g.nx, cap);
+  const int outer = h->g.ndim == 3 ? std::min(h->g.ny, h->g.nz) : 1;
+  while (w > (f32 ? 2 : 1) && (long long)h->g.Q * outer * ((h->g.nx + w - 1) / w) < 152) w /= 2;
+  return w;
 }
 
 bool shape_fits(mbo_ctx* h, const LaunchShape& c, int maxsm) {
@@ -758,11 +844,16 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
   cudaGetDevice(&h->dev);
   // launch shapes
   h->tx = pick_tx(g.nx, dtype == MBO_F32 ? 8 : 4);
-  // measured on GB300 (1024^2, n = 3): 192 threads best for FP32 rows, 128 for FP64
-  h->row_threads = g.nx >= 2048 ? 256
-                   : g.nx >= 1024 ? (dtype == MBO_F32 ? 192 : 128)
-                   : (g.nx >= 256 ? 128 : (g.nx >= 64 ? 64 : 32));
-  h->axis_threads = 256;
+  // measured on GB300 (1024^2, n = 3): 192 threads best for FP32 and FP64 rows.
+  // FP64 (168 registers: 384 threads fit on an SM): 192 from 256 points on (two
+  // blocks per SM at 1024, one round of butterflies at 256 - 648), 384 where a row
+  // fills the SM's shared memory, 128 for short rows (128^2, n = 2: 64 threads 26.6
+  // us, 128 threads 23.1 us)
+  if (dtype == MBO_F32)
+    h->row_threads = g.nx >= 2048 ? 256 : g.nx >= 1024 ? 192 : (g.nx >= 256 ? 128 : (g.nx >= 64 ? 64 : 32));
+  else
+    h->row_threads = row_smem_bytes(g, 8, false) > 114 * 1024 ? 384 : g.nx >= 256 ? 192 : g.nx >= 64 ? 128 : 32;
+  h->axis_threads = dtype == MBO_F32 ? 256 : 128;  // FP64: 168 registers, three blocks per SM
   if (dtype == MBO_F32) {
     // FP32 warp-plan strided passes, measured on GB300: 16-column tiles (one
     // 128-byte line per tile row) where an axis of 512 is strided (512^3:
@@ -819,7 +910,7 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
   }
   size_t rs = row_smem_bytes(g, h->elem, true);
   size_t as = 0;       // shared memory of the strided passes, each by its own plan
-  int min_tx = h->tx;  // narrowest column tile of any strided pass
+  int min_tx = std::min(h->tx, net_width(h, h->tx));  // narrowest column tile of any strided pass
   if (dtype == MBO_F32 && axis_plan(g, 0, true).lq) rs = std::max(rs, wrow_smem_bytes(g, g.nx, true));
   for (int ax = 1; ax < ndim; ++ax) {
     const int L = ax == 1 ? g.ny : g.nz;
@@ -850,8 +941,10 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
   const int rows = g.nz * g.ny;
   // the autotuner may narrow the column tiles (down to half, or 4 columns)
   if (c.autotune && !c.axis_tx) min_tx = std::max(1, std::min(min_tx, std::min(h->tx / 2, 4)));
-  const int tiles = g.Q * std::max(g.nz, g.ny) * (g.nx / min_tx);
-  const size_t nparts = (size_t)std::max(rows, tiles);
+  // outer rows of a strided pass: the other strided axis (none in 2-D)
+  const int tiles = g.Q * (ndim == 3 ? std::max(g.nz, g.ny) : 1) * ((g.nx + min_tx - 1) / min_tx);
+  // one slot per block that reduces: rows, column tiles, or one wave of 256 threads over the points
+  const size_t nparts = std::max<size_t>(std::max(rows, tiles), (size_t)std::min<long long>((g.P + 255) / 256, 152 * 8));
   h->ngroups = (nparts + kReduceGroup - 1) / kReduceGroup;
   // the small control arrays share one allocation
   size_t ctl_bytes = 0;

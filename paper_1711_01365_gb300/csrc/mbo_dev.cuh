@@ -372,6 +372,22 @@ template <typename R> __device__ __forceinline__ R polar2(const R* m, R* b, R& s
   const R rho2 = p * p + q * q, sig2 = r * r + t * t;
   const R rho = sqrt(rho2), sig = sqrt(sig2);
   smin = R(0.5) * fabs(rho - sig);
+  if constexpr (sizeof(R) == 8) {
+    // FP64 square roots and quotients are the long part of this point: one
+    // reciprocal square root of the larger sum does (in its normal range).  It
+    // ends within 1.5 ulp like the root, the quotient and the product below.
+    const R big = rho2 >= sig2 ? rho2 : sig2;
+    if (big > R(1e-280) && big < R(1e280)) {
+      const R inv = rsqrt(big);
+      const bool rot = rho2 >= sig2;
+      const R c = (rot ? p : r) * inv, s = (rot ? q : t) * inv;
+      b[0] = c;
+      b[1] = rot ? -s : s;
+      b[2] = s;
+      b[3] = rot ? c : -c;
+      return rot ? R(1) : R(-1);
+    }
+  }
   if (rho2 >= sig2) {
     if (rho2 > R(0)) {
       const R inv = R(1) / rho;
@@ -807,29 +823,9 @@ __device__ __forceinline__ R polar3_newton(const R* m, R* b, R& est, R skip_belo
   return polar_newton<3, ITMAX, NUN>(m, b, est, skip_below, cof2_floor);
 }
 
-// n = 3, FP32: the nearest matrix of the class sg (det = sg) through the
-// quaternion form of the problem (Horn 1987).  For a = sg m / |m|_F the
-// nearest rotation R(q) maximises tr(R^t a) = q^t K q over unit quaternions q,
-// K the symmetric traceless 4x4 matrix below, so q is the eigenvector of the
-// largest eigenvalue l1 = s1 + s2 + s3 (the singular values of a, the
-// smallest one signed by det a).  l1 is the largest root of
-//   p(l) = det(K - l I) = l^4 - 2 |a|^2 l^2 - 8 det(a) l + det K,
-// reached by Newton's method from the upper bound sqrt(3) |a|_F, and q is the
-// column of adj(K - l1 I) = prod_{i>1} (l_i - l1) q q^t with the largest
-// diagonal magnitude.  The other eigenvalues are s1 - s2 - s3, s2 - s1 - s3,
-// s3 - s1 - s2, so p'(l1) = 8 (s2 + s3)(s1 + s3)(s1 + s2): the eigenvector's
-// conditioning is that of the polar factor itself, 1 / (s2 + s3), and unlike
-// the Newton iteration nothing here inverts a; the rounding of l1, however,
-// enters q as eps / (s2 + s3)^2.  Returns p'(l1) / 32, a lower bound of
-// (s2 + s3) / |m|_F, for the caller's accuracy test.
-__device__ __forceinline__ float polar3_quat(const float* m, float sg, float* b) {
-  float n2 = 0.f;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) n2 += m[k] * m[k];
-  const float sc = sg * rsqrtf(n2);
-  float a[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) a[k] = m[k] * sc;
+// FP32 eigenvector (not normalised) of the largest eigenvalue l1 of K(a), for
+// |a|_F = 1 and det a >= 0.  Returns p'(l1) / 32.
+__device__ __forceinline__ float quat_vec(const float* a, float (&q)[4], float& l1) {
   float na = 0.f;
 #pragma unroll
   for (int k = 0; k < 9; ++k) na += a[k] * a[k];
@@ -890,6 +886,40 @@ __device__ __forceinline__ float polar3_quat(const float* m, float sg, float* b)
   if (M11 < best) { best = M11; w = -M01; x = M11; y = -M12; z = M13; }
   if (M22 < best) { best = M22; w = M02; x = -M12; y = M22; z = -M23; }
   if (M33 < best) { best = M33; w = -M03; x = M13; y = -M23; z = M33; }
+  q[0] = w;
+  q[1] = x;
+  q[2] = y;
+  q[3] = z;
+  l1 = lam;
+  return dp * (1.f / 32.f);
+}
+
+// n = 3, FP32: the nearest matrix of the class sg (det = sg) through the
+// quaternion form of the problem (Horn 1987).  For a = sg m / |m|_F the
+// nearest rotation R(q) maximises tr(R^t a) = q^t K q over unit quaternions q,
+// K the symmetric traceless 4x4 matrix below, so q is the eigenvector of the
+// largest eigenvalue l1 = s1 + s2 + s3 (the singular values of a, the
+// smallest one signed by det a).  l1 is the largest root of
+//   p(l) = det(K - l I) = l^4 - 2 |a|^2 l^2 - 8 det(a) l + det K,
+// reached by Newton's method from the upper bound sqrt(3) |a|_F, and q is the
+// column of adj(K - l1 I) = prod_{i>1} (l_i - l1) q q^t with the largest
+// diagonal magnitude.  The other eigenvalues are s1 - s2 - s3, s2 - s1 - s3,
+// s3 - s1 - s2, so p'(l1) = 8 (s2 + s3)(s1 + s3)(s1 + s2): the eigenvector's
+// conditioning is that of the polar factor itself, 1 / (s2 + s3), and unlike
+// the Newton iteration nothing here inverts a; the rounding of l1, however,
+// enters q as eps / (s2 + s3)^2.  Returns p'(l1) / 32, a lower bound of
+// (s2 + s3) / |m|_F, for the caller's accuracy test.
+__device__ __forceinline__ float polar3_quat(const float* m, float sg, float* b) {
+  float n2 = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) n2 += m[k] * m[k];
+  const float sc = sg * rsqrtf(n2);
+  float a[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) a[k] = m[k] * sc;
+  float q[4], l1;
+  const float gap = quat_vec(a, q, l1);
+  const float w = q[0], x = q[1], y = q[2], z = q[3];
   const float ww = w * w, xx = x * x, yy = y * y, zz = z * z;
   const float f = sg / (ww + xx + yy + zz);
   b[0] = (ww + xx - yy - zz) * f;
@@ -901,7 +931,7 @@ __device__ __forceinline__ float polar3_quat(const float* m, float sg, float* b)
   b[6] = 2.f * (x * z - w * y) * f;
   b[7] = 2.f * (y * z + w * x) * f;
   b[8] = (ww - xx - yy + zz) * f;
-  return dp * (1.f / 32.f);
+  return gap;
 }
 
 template <int NM, typename R> __device__ __forceinline__ R polar(const R* m, R* b, R& smin) {
@@ -1032,10 +1062,162 @@ static __device__ __noinline__ double polar4_jacobi(const double* m, double* b, 
   return want;
 }
 
+// n = 3, FP64: the polar factor from an FP32 quaternion refined in FP64.  FP64
+// instructions issue at 1/64 of the FP32 rate on this GPU, and the scaled Newton
+// iteration needs about 500 of them per point; here all but some 110 are FP32.
+//
+// For a = sg m, sg the sign of det m, the nearest rotation R(q) maximises
+// q^t K q over unit quaternions (Horn 1987; K as in polar3_quat), so q is the
+// eigenvector of the largest eigenvalue of the symmetric 4x4 matrix K.  With q
+// from polar3_quat_vec in FP32 (error about eps32 / gap), a correction step is
+//   r = K q - mu q (FP64, mu the Rayleigh quotient),  (K - mu) d = -r, d orthogonal to q,
+// whose matrix and solution only need a few digits: mu I - K + c q q^t is positive
+// definite for c > 0 (its smallest eigenvalue is the gap l1 - l2 = 2 (s2 + s3)),
+// factored once in FP32 and used by every step.  A step takes the error e to
+// about eps32 cond e, cond = |K| / gap: two steps reach FP64 rounding.  They stop
+// once d is at most kQuatSettled, when what is left is below rounding.
+//
+// Taken where the class and the eigenvector are clear in FP32: |det m| above
+// kQuatDet |m|^3 and the gap bound of the quaternion form at least kQuatGap64;
+// elsewhere (and out of the FP32 range) it returns false and the caller goes on
+// with Newton.  Against polar factors in extended precision its error is no
+// larger than the iteration's (about 4e-16 / gap each).
+constexpr float kQuatDet = 1e-4f;
+constexpr float kQuatGap64 = 0.02f;
+constexpr double kQuatSettled = 2e-11;
+
+__device__ __forceinline__ bool polar3_quat_f64(const double* m, double* b, double& sg) {
+  float f[9], n2 = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    f[k] = (float)m[k];
+    n2 += f[k] * f[k];
+  }
+  if (!(n2 > 1e-24f && n2 < 1e24f)) return false;  // out of range, or not finite
+  const float inv = rsqrtf(n2);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) f[k] *= inv;
+  const float det = f[0] * (f[4] * f[8] - f[5] * f[7]) - f[1] * (f[3] * f[8] - f[5] * f[6]) +
+                    f[2] * (f[3] * f[7] - f[4] * f[6]);
+  if (!(fabsf(det) > kQuatDet)) return false;
+  const float sf = det >= 0.f ? 1.f : -1.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) f[k] *= sf;
+  float v[4], l1;
+  if (!(quat_vec(f, v, l1) >= kQuatGap64)) return false;
+  sg = (double)sf;
+  {
+    const float in = rsqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] *= in;
+  }
+  // FP32 factor L D L^t of mu I - K + q q^t (K scaled to |a|_F = 1)
+  float l10, l20, l30, l21, l31, l32, d0, d1, d2, d3;
+  {
+    const float k00 = f[0] + f[4] + f[8], k11 = f[0] - f[4] - f[8], k22 = -f[0] + f[4] - f[8],
+                k33 = -f[0] - f[4] + f[8];
+    const float a00 = l1 - k00 + v[0] * v[0], a11 = l1 - k11 + v[1] * v[1], a22 = l1 - k22 + v[2] * v[2],
+                a33 = l1 - k33 + v[3] * v[3];
+    const float a10 = v[0] * v[1] - (f[7] - f[5]), a20 = v[0] * v[2] - (f[2] - f[6]),
+                a30 = v[0] * v[3] - (f[3] - f[1]), a21 = v[1] * v[2] - (f[1] + f[3]),
+                a31 = v[1] * v[3] - (f[2] + f[6]), a32 = v[2] * v[3] - (f[5] + f[7]);
+    d0 = __frcp_rn(a00);
+    l10 = a10 * d0, l20 = a20 * d0, l30 = a30 * d0;
+    const float b11 = a11 - l10 * a10, b21 = a21 - l20 * a10, b31 = a31 - l30 * a10;
+    const float b22 = a22 - l20 * a20, b32 = a32 - l30 * a20, b33 = a33 - l30 * a30;
+    d1 = __frcp_rn(b11);
+    l21 = b21 * d1, l31 = b31 * d1;
+    const float c22 = b22 - l21 * b21, c32 = b32 - l31 * b21, c33 = b33 - l31 * b31;
+    d2 = __frcp_rn(c22);
+    l32 = c32 * d2;
+    d3 = __frcp_rn(c33 - l32 * c32);
+  }
+  // K of sg m; the signs are flipped in the integer pipe
+  auto sgn = [neg = sf < 0.f](double x) {
+    return neg ? __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x)) : x;
+  };
+  const double t0 = sgn(m[0]), t4 = sgn(m[4]), t8 = sgn(m[8]);
+  const double p48 = t4 + t8, m48 = t4 - t8;
+  const double K00 = t0 + p48, K11 = t0 - p48, K22 = m48 - t0, K33 = -(t0 + m48);
+  const double K01 = sgn(m[7] - m[5]), K02 = sgn(m[2] - m[6]), K03 = sgn(m[3] - m[1]);
+  const double K12 = sgn(m[1] + m[3]), K13 = sgn(m[2] + m[6]), K23 = sgn(m[5] + m[7]);
+  double q[4] = {(double)v[0], (double)v[1], (double)v[2], (double)v[3]};
+  bool settled = false;
+#pragma unroll 1
+  for (int it = 0; it < 4; ++it) {
+    const double y0 = K00 * q[0] + K01 * q[1] + K02 * q[2] + K03 * q[3];
+    const double y1 = K01 * q[0] + K11 * q[1] + K12 * q[2] + K13 * q[3];
+    const double y2 = K02 * q[0] + K12 * q[1] + K22 * q[2] + K23 * q[3];
+    const double y3 = K03 * q[0] + K13 * q[1] + K23 * q[2] + K33 * q[3];
+    // mu only has to make r orthogonal to q up to the size of d: q q within
+    // 1e-6 of 1 would leave mu 1e-6 off, so divide by it (to first order: the
+    // norm is 1 + e with e below 1e-6, and e^2 is below rounding)
+    const double qq = q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
+    const double mu = (y0 * q[0] + y1 * q[1] + y2 * q[2] + y3 * q[3]) * (2.0 - qq);
+    const float r0 = (float)(y0 - mu * q[0]) * inv, r1 = (float)(y1 - mu * q[1]) * inv;
+    const float r2 = (float)(y2 - mu * q[2]) * inv, r3 = (float)(y3 - mu * q[3]) * inv;
+    const float z1 = r1 - l10 * r0;
+    const float z2 = r2 - l20 * r0 - l21 * z1;
+    const float z3 = r3 - l30 * r0 - l31 * z1 - l32 * z2;
+    const float x3 = z3 * d3;
+    const float x2 = z2 * d2 - l32 * x3;
+    const float x1 = z1 * d1 - l21 * x2 - l31 * x3;
+    const float x0 = r0 * d0 - l10 * x1 - l20 * x2 - l30 * x3;
+    q[0] += (double)x0;
+    q[1] += (double)x1;
+    q[2] += (double)x2;
+    q[3] += (double)x3;
+    const float dmax = fmaxf(fmaxf(fabsf(x0), fabsf(x1)), fmaxf(fabsf(x2), fabsf(x3)));
+    if (dmax <= (float)kQuatSettled) {
+      settled = true;
+      break;
+    }
+  }
+  if (!settled) return false;
+  const double ww = q[0] * q[0], xx = q[1] * q[1], yy = q[2] * q[2], zz = q[3] * q[3];
+  const double wx = ww + xx, yz = yy + zz;
+  // sg / |q|^2: |q|^2 = 1 + e with |e| of the FP32 rounding, so 1 - e + e^2 is exact to rounding
+  const double e = (wx + yz) - 1.0;
+  const double g = sgn((1.0 - e) + e * e), h = g + g;
+  const double wmx = ww - xx, ymz = yy - zz;
+  b[0] = (wx - yz) * g;
+  b[4] = (wmx + ymz) * g;
+  b[8] = (wmx - ymz) * g;
+  const double hx = h * q[1], hy = h * q[2], hz = h * q[3];
+  const double xy = hx * q[2], xz = hx * q[3], yz2 = hy * q[3];
+  b[1] = xy - hz * q[0];
+  b[3] = xy + hz * q[0];
+  b[2] = xz + hy * q[0];
+  b[6] = xz - hy * q[0];
+  b[5] = yz2 - hx * q[0];
+  b[7] = yz2 + hx * q[0];
+  return true;
+}
+
+// n = 3: Newton, then the Jacobi construction where m is singular to working
+// precision; out of line, for the points polar3_quat_f64 leaves.
+struct MatD9 {
+  double b[9];
+  double sg;
+};
+static __device__ __noinline__ MatD9 polar3_newton_cold(const double* m) {
+  MatD9 r;
+  double x[9], nx = 0.0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    x[k] = m[k];
+    nx += x[k] * x[k];
+  }
+  double est = 0.0, smin;
+  r.sg = polar3_newton<16, 3>(x, r.b, est, 1e-12 * sqrt(nx), 1e-24 * nx * nx);
+  if (!(est > 1e-12 * sqrt(nx))) r.sg = polar3(x, r.b, smin);
+  return r;
+}
+
 // FP64 projection used by the FP64 path and by the FP32 path's
-// re-projection: Newton, and the one-sided Jacobi construction for matrices
+// re-projection: for n = 3 the refined quaternion form, else and elsewhere Newton, and the one-sided Jacobi construction for matrices
 // that are singular to working precision (rank-deficient ties included).
-template <int NM> __device__ __forceinline__ double polar_f64(const double* m, double* b, double& smin) {
+template <int NM> __device__ __forceinline__ double polar_f64(const double* m, double* b) {
   if constexpr (NM == 4) {
     double nx = 0.0;
 #pragma unroll
@@ -1047,35 +1229,35 @@ template <int NM> __device__ __forceinline__ double polar_f64(const double* m, d
     if (nx > 1e-30 && nx < 1e30 && d * d > 1e-26 * nx * nx * nx * nx && fabs(d) > 1e-18) {
       double est = 0.0;
       const double sg = polar_newton<4, 16, 3>(m, b, est, 1e-12 * sqrt(nx), 1e-24 * nx * nx * nx);
-      smin = est;
       if (est > 1e-12 * sqrt(nx)) return sg;
     }
+    double smin;
     return polar4_jacobi(m, b, smin);
   } else if constexpr (NM == 3) {
-    double nx = 0.0;
+    double sg;
+    if (polar3_quat_f64(m, b, sg)) return sg;
+    const MatD9 r = polar3_newton_cold(m);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) nx += m[k] * m[k];
-    double est = 0.0;
-    const double sg = polar3_newton<16, 3>(m, b, est, 1e-12 * sqrt(nx), 1e-24 * nx * nx);
-    smin = est;
-    if (est > 1e-12 * sqrt(nx)) return sg;
-    return polar3(m, b, smin);
+    for (int k = 0; k < 9; ++k) b[k] = r.b[k];
+    return r.sg;
   } else {
+    double smin;
     return polar<NM>(m, b, smin);
   }
 }
 
+template <int NM, typename R> __device__ __forceinline__ R det_value(const R* m) {
+  if constexpr (NM == 1) return m[0];
+  else if constexpr (NM == 2) return m[0] * m[3] - m[1] * m[2];
+  else if constexpr (NM == 3)
+    return m[0] * (m[4] * m[8] - m[5] * m[7]) - m[1] * (m[3] * m[8] - m[5] * m[6]) +
+           m[2] * (m[3] * m[7] - m[4] * m[6]);
+  else
+    return det4(m);
+}
 // Sign of det of an (orthogonal) matrix: +1 / -1.
 template <int NM, typename R> __device__ __forceinline__ R det_sign(const R* m) {
-  R d;
-  if constexpr (NM == 1) d = m[0];
-  else if constexpr (NM == 2) d = m[0] * m[3] - m[1] * m[2];
-  else if constexpr (NM == 3)
-    d = m[0] * (m[4] * m[8] - m[5] * m[7]) - m[1] * (m[3] * m[8] - m[5] * m[6]) +
-        m[2] * (m[3] * m[7] - m[4] * m[6]);
-  else
-    d = det4(m);
-  return d >= R(0) ? R(1) : R(-1);
+  return det_value<NM>(m) >= R(0) ? R(1) : R(-1);
 }
 
 // ---------------------------------------------------------------------------

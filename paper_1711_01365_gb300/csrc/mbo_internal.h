@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace mbo {
 
 constexpr int kMaxStages = 8;
@@ -33,6 +35,16 @@ struct Stage {
   FastDiv dm;   // division by m
   FastDiv dnr;  // division by N / rad
 };
+
+// A twiddle of the FP64 passes' fixed-point transforms (mbo_fixed.cuh): cos and
+// -sin in Q60, each (h 2^31 + l) / 2^60 with 0 <= l < 2^31.  As large as the
+// complex FP64 value it stands for.
+struct alignas(16) FxTw {
+  int ch, cl, sh, sl;
+};
+inline __host__ __device__ FxTw fx_tw(long long c, long long s) {
+  return FxTw{(int)(c >> 31), (int)(c & 0x7fffffff), (int)(s >> 31), (int)(s & 0x7fffffff)};
+}
 
 // Transform plan of one axis.
 //   lq == 0: the in-place network of nst stages (forward stages applied in
@@ -125,7 +137,7 @@ __host__ __device__ inline float col_weight(const Geom& g, int q, int kx) {
 
 // Per-axis tables in the element type R (0 = x, 1 = y, 2 = z).
 template <typename R> struct Tables {
-  const void* tw[3];   // per-stage twiddles of each axis (see Stage::tw)
+  const void* tw[3];   // per-stage twiddles of each axis (see Stage::tw): complex R, FxTw in FP64
   const R* g[3];       // exp(-4 pi^2 tau k^2), k the signed frequency held at each
                        // spectrum position of the forward transform (digit-reversed
                        // or natural, per the axis plan)
@@ -212,12 +224,15 @@ cudaError_t launch_project(const Geom& g, const R* At, R* B, int8_t* det_sign,
 // Plan helpers (mbo_api.cu).
 bool factor23(int64_t N, int& a, int& b);
 FastDiv make_div(unsigned d);
-Plan make_plan(int N);
+// small_code: radices up to 9 only
+Plan make_plan(int N, bool small_code = false);
 // Plan of one axis of a geometry: the warp-cooperative plan (FP32, lengths
 // 256, 512, 768, 1024, 1536, 2048; strided axes need nx % 4 == 0) where one
 // exists, else make_plan.
 Plan axis_plan(const Geom& g, int axis, bool f32);
 int plan_twiddles(const Plan& p);
+// pos[k]: position where the forward transform of a plan leaves frequency k.
+void digit_positions(const Plan& p, int N, std::vector<int>& pos);
 int pick_tx(int nx, int cap);
 // Columns per tile of the network strided passes: `cap` (64 bytes a tile row),
 // or the power of two that covers a narrower field.
@@ -235,6 +250,9 @@ size_t wcol_smem_bytes(int L, int tx, int stages);
 cudaError_t launch_wrow(RowMode mode, const Geom& g, const Tables<float>& t, const float* A_in,
                         float* A_out, void* W, const StatsPtrs& sp, double fallback_sigma,
                         cudaStream_t s, bool prepare_only);
+// The projecting pass with helper warps (k_wsmall.cu), for grids of at most two blocks per SM.
+cudaError_t launch_wrow_small(const Geom& g, const Tables<float>& t, float* A, void* W, const StatsPtrs& sp,
+                              float fb, int blocks, size_t smem, cudaStream_t s, bool prepare_only);
 cudaError_t launch_wcol(AxisMode mode, int axis, const Geom& g, const Tables<float>& t, void* W,
                         const StatsPtrs& sp, int tx, cudaStream_t s, bool prepare_only,
                         const CUtensorMap* tm, int stages, const void* l2_hint = nullptr,

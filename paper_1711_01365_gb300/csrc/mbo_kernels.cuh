@@ -66,11 +66,11 @@ template <int NM> __device__ __noinline__ ProjV<NM> quat_cold(MatV<NM> m, float 
 
 template <int NM> __device__ __noinline__ ProjV<NM> f64_cold(MatV<NM> m) {
   constexpr int C = NM * NM;
-  double md[C], bd[C], sd;
+  double md[C], bd[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) md[c] = (double)m.v[c];
   ProjV<NM> r;
-  r.sg = (float)polar_f64<NM>(md, bd, sd);
+  r.sg = (float)polar_f64<NM>(md, bd);
 #pragma unroll
   for (int c = 0; c < C; ++c) r.b[c] = (float)bd[c];
   r.gap = 0.f;
@@ -93,8 +93,7 @@ constexpr float kQuatGap = 0.05f;
 template <int NM, typename R>
 __device__ __forceinline__ bool project_point(const R* m, R* b, R& sg, R fb) {
   if constexpr (sizeof(R) == 8) {
-    double sm;
-    sg = polar_f64<NM>(m, b, sm);
+    sg = polar_f64<NM>(m, b);
     return true;
   } else if constexpr (NM >= 3) {
     float nx = 0.f;
@@ -152,8 +151,7 @@ __device__ __forceinline__ R project_point_f64(const R* m, R* b) {
     for (int c = 0; c < C; ++c) b[c] = r.b[c];
     return r.sg;
   } else {
-    double sd;
-    return polar_f64<NM>(m, b, sd);
+    return polar_f64<NM>(m, b);
   }
 }
 
@@ -164,14 +162,42 @@ __device__ __forceinline__ void finish_point(R* __restrict__ A, long long P, lon
                                              const R* old, const R* b, R sg, V* dst, int qstride,
                                              PointStats<R>& ps) {
   constexpr int C = NM * NM, Q = (C + 1) / 2;
-  R d = R(0), nb = R(0);
+  R nb = R(0);
+  if constexpr (sizeof(R) == 8) {
+    // FP64 compares and the old field's determinant would cost as much as the
+    // projection: the bits of |delta| compare as integers (NaN, above every
+    // number, is passed over as fmax does), and an orthogonal matrix has its
+    // determinant's sign in FP32
+    unsigned long long mx = (unsigned long long)__double_as_longlong(ps.maxd);
 #pragma unroll
-  for (int c = 0; c < C; ++c) {
-    d = fmax(d, fabs(b[c] - old[c]));
-    nb += b[c] * b[c];
+    for (int c = 0; c < C; ++c) {
+      const unsigned long long u =
+          (unsigned long long)__double_as_longlong(b[c] - old[c]) & 0x7fffffffffffffffull;
+      mx = (u > mx && u <= 0x7ff0000000000000ull) ? u : mx;
+      nb += b[c] * b[c];
+    }
+    ps.maxd = __longlong_as_double((long long)mx);
+    float of[C], big = 0.f;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      of[c] = (float)old[c];
+      big = fmaxf(big, fabsf(of[c]));
+    }
+    const float df = det_value<NM>(of);
+    R so;
+    if (fabsf(df) > 0.25f && big < 2.f) so = df > 0.f ? R(1) : R(-1);
+    else so = det_sign<NM>(old);
+    ps.flips += (so != sg) ? 1 : 0;
+  } else {
+    R d = R(0);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      d = fmax(d, fabs(b[c] - old[c]));
+      nb += b[c] * b[c];
+    }
+    ps.maxd = fmax(ps.maxd, d);
+    ps.flips += (det_sign<NM>(old) != sg) ? 1 : 0;
   }
-  ps.maxd = fmax(ps.maxd, d);
-  ps.flips += (det_sign<NM>(old) != sg) ? 1 : 0;
   ps.defect += R(NM) - nb;
 #pragma unroll
   for (int c = 0; c < C; ++c) A[c * P + off + x] = b[c];
@@ -623,14 +649,6 @@ __device__ __forceinline__ R class_pair_checked(const R* m, R* tp, R* tm, R& dE,
   return smin;
 }
 
-template <int NM, typename R> __device__ __forceinline__ R det_value(const R* m) {
-  if constexpr (NM == 1) return m[0];
-  else if constexpr (NM == 2) return m[0] * m[3] - m[1] * m[2];
-  else
-    return m[0] * (m[4] * m[8] - m[5] * m[7]) - m[1] * (m[3] * m[8] - m[5] * m[6]) +
-           m[2] * (m[3] * m[7] - m[4] * m[6]);
-}
-
 // keys[x] = desc_key(dE(x)) for the diffused field At.  SELECT: the same pass
 // counts the points of A with det A(x) > 0 (where n_plus < 0 asks for that
 // number) and runs the first pass of the selection, so that neither reads a
@@ -945,6 +963,12 @@ template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>
   return e;
 }
 
+#define MBO_INSTANTIATE_POINTS(R)                                                              \
+  template cudaError_t launch_project<R>(const Geom&, const R*, R*, int8_t*, double,          \
+                                         cudaStream_t);                                        \
+  template cudaError_t launch_volume<R>(VolumePass, const Geom&, const R*, R*, unsigned long long*, \
+                                        SelectState*, const StatsPtrs&, double, int,           \
+                                        cudaStream_t, long long);
 #define MBO_INSTANTIATE(R)                                                                     \
   template cudaError_t prepare_kernels<R>(const Geom&, const Tables<R>&, int, int, int);       \
   template cudaError_t launch_row<R>(RowMode, const Geom&, const Tables<R>&, const R*, R*,     \
@@ -952,10 +976,6 @@ template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>
   template cudaError_t launch_axis<R>(AxisMode, int, const Geom&, const Tables<R>&, void*,     \
                                       const StatsPtrs&, int, int, cudaStream_t,                \
                                       const CUtensorMap*, int, const void*, long long);        \
-  template cudaError_t launch_project<R>(const Geom&, const R*, R*, int8_t*, double,          \
-                                         cudaStream_t);                                        \
-  template cudaError_t launch_volume<R>(VolumePass, const Geom&, const R*, R*, unsigned long long*, \
-                                        SelectState*, const StatsPtrs&, double, int,           \
-                                        cudaStream_t, long long);
+  MBO_INSTANTIATE_POINTS(R)
 
 }  // namespace mbo

@@ -60,7 +60,12 @@ __global__ void k_noalloc_tables(Plan pl, int N, int ntw, double tau, typename V
           const long long e = ((long long)n1 * j) % s.lb;
           double sn, cs;
           sincospi(2.0 * (double)e / (double)s.lb, &sn, &cs);
-          tw[i] = V{(R)cs, (R)(-sn)};
+          if constexpr (sizeof(R) == 8) {  // Q60 limbs of the fixed-point transforms
+            *reinterpret_cast<FxTw*>(&tw[i]) =
+                fx_tw(__double2ll_rn(cs * 0x1p60), __double2ll_rn(-sn * 0x1p60));
+          } else {
+            tw[i] = V{(R)cs, (R)(-sn)};
+          }
         }
       }
     }

@@ -108,3 +108,47 @@ def test_network_radices_and_ragged_tiles(M, dims, dtype):
     scaleE = float((F.abs().square().sum() / P + A.double().square().sum())) / (P * tau)
     assert abs(h.lyapunov(A) - E) <= (1e-5 if dtype == "f32" else 1e-12) * scaleE
     h.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4])
+@pytest.mark.parametrize("dims", [(2, 2), (3, 16), (6, 1536), (9, 2048), (2048, 2), (18, 54, 12), (1024, 1024)])
+@pytest.mark.parametrize("scale", [1.0, 1e-200, 1e200, 1e-320])
+def test_fixed_point_diffusion_is_scale_free(M, dims, n, scale):
+    """The FP64 transforms run in fixed point on a scale of their own per sequence: any finite magnitude,
+    one channel far below its partner, one bright point, constant fields; and a non-finite value still
+    reaches what a floating-point transform would make of it."""
+    if scale != 1.0 and np.prod(dims) > 50000:
+        pytest.skip("sizes are covered at scale 1")
+    if n == 4 and dims[-1] == 2048:
+        pytest.skip("rows of eight FP64 planes exceed the shared memory")
+    tau = 3.0 / max(dims) ** 2
+    g = torch.Generator(device="cuda").manual_seed(11)
+    A = torch.randn((n * n,) + dims, generator=g, device="cuda", dtype=torch.float64)
+    A[0] += 3.0
+    A.view(n * n, -1)[-1, 5 % A[0].numel()] = 1e4
+    if n > 1:
+        A[1] *= 1e-9
+        A[2] = 0.75
+    e = 0.0
+    for ax, N in enumerate(dims):
+        k = torch.fft.fftfreq(N, 1.0 / N, device="cuda", dtype=torch.float64)
+        e = e - 4 * np.pi ** 2 * tau * (k * k).reshape([-1 if ax == b else 1 for b in range(len(dims))])
+    d = tuple(range(1, len(dims) + 1))
+    want = torch.fft.ifftn(torch.fft.fftn(A, dim=d) * torch.exp(e), dim=d).real
+    h = M.Mbo(dims, n, tau, "f64")
+    out = torch.empty_like(A)
+    h.diffuse(A * scale, out)
+    if scale == 1e-320:  # denormals keep no digits: nothing but their size is asked
+        assert float(out.abs().max()) <= 1e-310
+    else:
+        rms = want.square().mean(dim=d, keepdim=True).sqrt()
+        pair = torch.maximum(rms[0::2], torch.cat([rms[1::2], rms[-1:]])[: rms[0::2].shape[0]])
+        lim = 3e-15 * torch.repeat_interleave(pair, 2, dim=0)[: n * n] * np.log2(A[0].numel() + 2)
+        assert bool(((out / scale - want).abs() <= lim).all())
+    bad = A.clone()
+    bad.view(n * n, -1)[0, 3 % A[0].numel()] = float("nan") if n % 2 else float("inf")
+    h.diffuse(bad, out)
+    assert not bool(torch.isfinite(out[0]).any())
+    if n > 2:
+        assert bool(torch.isfinite(out[2:]).all())  # the other planes are not touched
+    h.close()
