@@ -47,6 +47,8 @@
 #include "mbo_internal.h"
 #include "mbo_kernels.cuh"
 
+#include "mbo_box.cuh"
+
 namespace mbo {
 namespace {
 
@@ -75,8 +77,13 @@ template <typename T> struct SpreadArgs {
   const int* gsrc;       // group -> first source (ngroups + 1)
   const int* gt0;        // group -> footprint start in the bin tile, t0x | t0y << 4 | t0z << 8
   const int* bgrp;       // bin -> first group (nbins + 1)
+  // k_spread7: groups over the whole grid instead of per bin
+  const int4* g0;        // group -> footprint start on the grid (x, y even; z)
+  const int* seg;        // segment -> first group (nseg + 1)
+  int nseg;
   const int* bid;        // bin -> bin id (bz nb + by) nb + bx
-  T* F;                  // grid, C x nf^3
+  T* F;                  // grid box, C channels
+  GridBox box;
   long long nq;
   int C, nf, nb, W;
   T beta;
@@ -102,6 +109,41 @@ template <int WT> __device__ __forceinline__ int swz(int x, int y) {
   if constexpr (WT == 7) return x ^ (((y >> 1) & 1) << 3);
   return x;
 }
+// Add a block's tile ([c][z][y][x]) to the grid box.
+template <typename T, int WT>
+__device__ __forceinline__ void spread_flush(const SpreadArgs<T>& a, const T* tile, int c0, int cg, int W,
+                                             int TX, int TZ, int threads) {
+  const int b = a.bid[blockIdx.x];
+  const int bx = b % a.nb, by = (b / a.nb) % a.nb, bz = b / (a.nb * a.nb);
+  const int nf = a.nf;
+  const long long P = a.box.points();
+  const int lx = (bx * kBin - W / 2 + nf) % nf, ly = (by * kBin - W / 2 + nf) % nf,
+            lz = (bz * kBin - W / 2 + nf) % nf;
+  const int TV = TX * TX * TZ;
+  // sixteen lanes per tile row (TX is at most 17)
+  const int half = threadIdx.x & 15;
+  for (int row = threadIdx.x >> 4; row < cg * TZ * TX; row += threads / 16) {
+    const int c = row / (TZ * TX), zy = row - c * TZ * TX, z = zy / TX, y = zy - z * TX;
+    int gy = ly + y, gz = lz + z;
+    gy -= gy >= nf ? nf : 0;
+    gz -= gz >= nf ? nf : 0;
+    gy -= a.box.b0[1];
+    gz -= a.box.b0[2];
+    // tile rows outside the box hold zeros
+    if ((unsigned)gy >= (unsigned)a.box.bn[1] || (unsigned)gz >= (unsigned)a.box.bn[2]) continue;
+    T* Frow = a.F + (long long)(c0 + c) * P + ((long long)gz * a.box.bn[1] + gy) * a.box.bn[0];
+    const T* trow = tile + c * TV + zy * TX;
+    for (int x = half; x < TX; x += 16) {
+      const T v = trow[swz<WT>(x, y)];
+      if (v == T(0)) continue;
+      int gx = lx + x;
+      gx -= gx >= nf ? nf : 0;
+      gx -= a.box.b0[0];
+      if ((unsigned)gx < (unsigned)a.box.bn[0]) atomicAdd(&Frow[gx], v);
+    }
+  }
+}
+
 constexpr int kWS = 9;     // weight slots of x and of y per source (>= W + 1)
 constexpr int kWSrc = 28;  // per source: z[8] | x[kWS] | y[kWS] | 2 pad, then strengths
 template <typename T> __host__ __device__ constexpr int src_stride() { return sizeof(T) == 4 ? 44 : 34; }
@@ -207,42 +249,175 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs<T> a) {
   }
   __syncthreads();
 
-  // add the tile to the periodic grid: one warp per tile row
-  const int b = a.bid[blockIdx.x];
-  const int bx = b % a.nb, by = (b / a.nb) % a.nb, bz = b / (a.nb * a.nb);
-  const int nf = a.nf;
-  const long long P = (long long)nf * nf * nf;
-  const int lx = (bx * kBin - W / 2 + nf) % nf, ly = (by * kBin - W / 2 + nf) % nf,
-            lz = (bz * kBin - W / 2 + nf) % nf;
-  for (int row = warp; row < cg * TZ * TX; row += kSpreadThreads / 32) {
-    const int c = row / (TZ * TX), zy = row - c * TZ * TX, z = zy / TX, y = zy - z * TX;
-    int gy = ly + y, gz = lz + z;
-    gy -= gy >= nf ? nf : 0;
-    gz -= gz >= nf ? nf : 0;
-    T* Frow = a.F + (long long)(c0 + c) * P + ((long long)gz * nf + gy) * nf;
-    const T* trow = tile + c * TV + zy * TX;
-    for (int x = lane; x < TX; x += 32) {
-      const T v = trow[swz<WT>(x, y)];
-      if (v == T(0)) continue;
-      int gx = lx + x;
-      gx -= gx >= nf ? nf : 0;
-      atomicAdd(&Frow[gx], v);
+  spread_flush<T, WT>(a, tile, c0, cg, W, TX, TZ, kSpreadThreads);
+}
+
+// FP32, width 7 (eps = 1e-6, the paper's choice).  The work is the rank-one
+// update of a group's 64 footprint columns by 7 x CG values per source: FMA
+// work, so the kernel is laid out to keep the FMA pipe the limit.
+//   - Groups hold about 18 sources on the paper's sphere, so adding a group's
+//     7 x 8 x 8 x CG sums anywhere costs more than making them.  A warp takes a
+//     segment of a column of groups (one footprint start in x and y over the
+//     whole grid, z ascending, up to kSegSources sources) and slides its seven
+//     accumulator planes along z: only the plane that falls out leaves, straight
+//     to the grid box by reductions in L2 (eight neighbours along x share a
+//     sector), with no tile in shared memory and no block to wait for.
+//   - Two warps share a segment, one for each half of the 64 columns, and stage
+//     64 sources together: 16 warps per SM at 128 registers (one warp with both
+//     halves in its registers, 8 per SM, waited on instruction latency: 1.09 ms).
+//   - Packed two-lane multiply-adds over channel pairs: the z weights are stored
+//     twice so that a 16-byte load brings two packed operands; (w_x w_y) scales
+//     the strengths once per column.  54 instructions per source and half instead
+//     of 84.  The next source's operands are loaded while this one is summed.
+// Unit sphere of the paper (3.3M points, n = 3): 1.71 ms with a group per warp and a
+// shared-memory tile per bin, 0.84 ms (segments of 512 sources 0.86, 1024 0.94).
+constexpr int kSpread7Threads = 64;
+constexpr int kSegSources = 256;
+template <int CG> struct Spread7 {
+  static constexpr int NP = (CG + 1) / 2;                 // channel pairs
+  static constexpr int SP = (2 * NP + 3) / 4 * 4;         // strengths, padded to vectors
+  static constexpr int OX = 16 + SP, OY = OX + 8;         // z (twice, 14 + 2) | strengths | x | y
+  static constexpr int SRC = (OY + 8) / 4 % 2 ? OY + 8 : OY + 12;  // odd number of vectors: no bank conflicts
+};
+// Coordinate of the box from a footprint coordinate in [-W, nf + W).
+__device__ __forceinline__ int box_coord(int g, int nf, int b0) {
+  g += g < 0 ? nf : 0;
+  g -= g >= nf ? nf : 0;
+  return g - b0;
+}
+template <int CG>
+__global__ void __launch_bounds__(kSpread7Threads, 8) k_spread7(SpreadArgs<float> a) {
+  using S = Spread7<CG>;
+  constexpr int NP = S::NP;
+  __shared__ __align__(16) float stg[kSpread7Threads * S::SRC];
+  const int c0 = blockIdx.y * CG;
+  const int cg = min(CG, a.C - c0);
+  const int tid = threadIdx.x;
+  const int i = tid & 7, j = tid >> 3;  // footprint column
+  int g = a.seg[blockIdx.x];
+  const int ge = a.seg[blockIdx.x + 1];
+  const int4 start = a.g0[g];
+  int tz = start.z;
+  const long long P = a.box.points(), plane = (long long)a.box.bn[0] * a.box.bn[1];
+  const int gx = box_coord(start.x + i, a.nf, a.box.b0[0]);
+  float* F = a.F + c0 * P + (long long)box_coord(start.y + j, a.nf, a.box.b0[1]) * a.box.bn[0] + gx;
+  float2 acc[7][NP];
+#pragma unroll
+  for (int k = 0; k < 7; ++k)
+#pragma unroll
+    for (int c = 0; c < NP; ++c) acc[k][c] = make_float2(0.f, 0.f);
+  // the lowest plane to the grid, the others down by one
+  auto slide = [&]() {
+    const long long at = box_coord(tz, a.nf, a.box.b0[2]) * plane;
+#pragma unroll
+    for (int c = 0; c < CG; ++c) {
+      if (c < cg) atomicAdd(F + c * P + at, c % 2 ? acc[0][c / 2].y : acc[0][c / 2].x);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+#pragma unroll
+      for (int c = 0; c < NP; ++c) acc[k][c] = acc[k + 1][c];
+#pragma unroll
+    for (int c = 0; c < NP; ++c) acc[6][c] = make_float2(0.f, 0.f);
+    ++tz;
+  };
+  const int s1 = a.gsrc[ge];
+  int gend = a.gsrc[g + 1];  // the end of the group in work
+  for (int cs = a.gsrc[g]; cs < s1; cs += kSpread7Threads) {
+    const int ns = min(kSpread7Threads, s1 - cs);
+    __syncthreads();
+    if (tid < ns) {
+      const V4<float> u = a.su[cs + tid];  // distance past the group footprint start
+      const long long src = a.sidx[cs + tid];
+      float st[S::SP];
+#pragma unroll
+      for (int c = 0; c < S::SP; ++c) st[c] = c < CG && c < cg ? a.A[(long long)(c0 + c) * a.nq + src] * u.w : 0.f;
+      float4* dst = reinterpret_cast<float4*>(stg + tid * S::SRC);
+      constexpr float sc2 = 2.f / 7.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float za = es_kernel((float(2 * k) - u.z) * sc2, a.beta);
+        const float zb = 2 * k + 1 < 7 ? es_kernel((float(2 * k + 1) - u.z) * sc2, a.beta) : 0.f;
+        dst[k] = make_float4(za, za, zb, zb);
+      }
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        float x[4], y[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          x[e] = es_kernel((float(4 * v + e) - u.x) * sc2, a.beta);
+          y[e] = es_kernel((float(4 * v + e) - u.y) * sc2, a.beta);
+        }
+        dst[S::OX / 4 + v] = make_float4(x[0], x[1], x[2], x[3]);
+        dst[S::OY / 4 + v] = make_float4(y[0], y[1], y[2], y[3]);
+      }
+#pragma unroll
+      for (int v = 0; v < S::SP / 4; ++v) dst[4 + v] = make_float4(st[4 * v], st[4 * v + 1], st[4 * v + 2], st[4 * v + 3]);
+    }
+    __syncthreads();
+    float4 z[4], sv[S::SP / 4];
+    float wx, wy;
+    auto fetch = [&](int q) {
+      const float4* r = reinterpret_cast<const float4*>(stg + q * S::SRC);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) z[v] = r[v];
+#pragma unroll
+      for (int v = 0; v < S::SP / 4; ++v) sv[v] = r[4 + v];
+      const float* w = stg + q * S::SRC;
+      wx = w[S::OX + i];
+      wy = w[S::OY + j];
+    };
+    fetch(0);
+    int q = 0;
+    while (q < ns) {
+      if (cs + q == gend) {  // the next group of the column, some planes up
+        ++g;
+        gend = a.gsrc[g + 1];
+        const int up = a.g0[g].z;
+#pragma unroll 1
+        while (tz < up) slide();
+      }
+      const int qe = min(ns, gend - cs);
+      for (; q < qe; ++q) {
+        const float2 zz[7] = {{z[0].x, z[0].y}, {z[0].z, z[0].w}, {z[1].x, z[1].y}, {z[1].z, z[1].w},
+                              {z[2].x, z[2].y}, {z[2].z, z[2].w}, {z[3].x, z[3].y}};
+        const float w = wx * wy;
+        float2 pc[NP];
+#pragma unroll
+        for (int c = 0; c < NP; ++c) {
+          const float4 v = sv[c / 2];
+          const float2 t = c % 2 ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+          pc[c] = __fmul2_rn(t, make_float2(w, w));
+        }
+        if (q + 1 < ns) fetch(q + 1);
+#pragma unroll
+        for (int k = 0; k < 7; ++k)
+#pragma unroll
+          for (int c = 0; c < NP; ++c) acc[k][c] = __ffma2_rn(zz[k], pc[c], acc[k][c]);
+      }
     }
   }
+#pragma unroll 1
+  for (int k = 0; k < 7; ++k) slide();
 }
 
 template <typename T> struct InterpArgs {
-  const T* F;          // grid, C x nf^3
+  const T* F;          // grid box, C channels
+  GridBox box;
   const V4<T>* tu;     // targets sorted by group: d per axis
   const int* tidx;     // target -> field point
   const int* tgrp;     // group -> first target (ngroups + 1)
   const int4* tg0;     // group -> first footprint point on the grid (gx, gy, gz)
-  T* dst;              // C x nq: out[c][tidx[t]] (diffuse) or scratch[c][t] (step)
+  T* dst;              // C x nq, the caller's order: the passes that follow stream it
   long long nq;
   int nf, W;
-  bool scatter;        // write at tidx[t] (true) or at t (false)
   T beta;
 };
+
+// Offset of a grid point of the box.
+__device__ __forceinline__ long long box_at(const GridBox& b, int gx, int gy, int gz) {
+  return ((long long)(gz - b.b0[2]) * b.bn[1] + (gy - b.b0[1])) * b.bn[0] + (gx - b.b0[0]);
+}
 
 // One block per target group: the group's W^3 footprint values (C channels
 // padded to CP, point-major) are staged in shared memory once; each thread
@@ -258,7 +433,7 @@ __global__ void __launch_bounds__(kInterpBlock) k_interp(InterpArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* fp = reinterpret_cast<T*>(smem_raw);  // [W^3][CP]
   const int W = WT ? WT : a.W, W2 = W * W, W3 = W2 * W, nf = a.nf;
-  const long long P = (long long)nf * nf * nf;
+  const long long P = a.box.points();
   const int g = blockIdx.x;
   const int4 g0 = a.tg0[g];
   for (int e = threadIdx.x; e < CP * W3; e += kInterpBlock) {
@@ -270,7 +445,7 @@ __global__ void __launch_bounds__(kInterpBlock) k_interp(InterpArgs<T> a) {
       gx -= gx >= nf ? nf : 0;
       gy -= gy >= nf ? nf : 0;
       gz -= gz >= nf ? nf : 0;
-      v = __ldg(&a.F[c * P + ((long long)gz * nf + gy) * nf + gx]);
+      v = __ldg(&a.F[c * P + box_at(a.box, gx, gy, gz)]);
     }
     fp[p * CP + c] = v;
   }
@@ -325,36 +500,162 @@ __global__ void __launch_bounds__(kInterpBlock) k_interp(InterpArgs<T> a) {
         }
       }
     }
-    const long long q = a.scatter ? (long long)a.tidx[t] : (long long)t;
+    const long long q = a.tidx[t];
 #pragma unroll
     for (int c = 0; c < C; ++c) a.dst[c * a.nq + q] = acc[c];
   }
 }
 
+// FP32, width 7, n = 2 and 3: a lane evaluates two targets at once, so a
+// footprint point (broadcast from shared memory, whose bandwidth bounds this
+// kernel: a 16-byte broadcast moves 512 bytes to the warp) serves both; channels
+// in pairs, by packed multiply-adds.  A warp takes 64 targets of its group at a
+// time, or 32 where no more are left.  Unit sphere of the paper: one target per lane
+// 0.79 ms, two 0.645 ms.
+template <int NM> struct Interp7 {
+  static constexpr int C = NM * NM, NP = (C + 1) / 2, ST = (2 * NP + 3) / 4 * 4;  // floats per point
+};
+template <int NM, int NT>
+__device__ __forceinline__ void interp7_targets(const InterpArgs<float>& a, const float* fp, int t, int t1) {
+  using S = Interp7<NM>;
+  constexpr float sc2 = 2.f / 7.f;
+  float2 wx[NT][7], acc[NT][S::NP];
+  float wy[NT][7], uz[NT];
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+    const V4<float> u = a.tu[min(t + 32 * n, t1 - 1)];
+    uz[n] = u.z;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      const float w = es_kernel((float(i) - u.x) * sc2, a.beta);
+      wx[n][i] = make_float2(w, w);
+      wy[n][i] = es_kernel((float(i) - u.y) * sc2, a.beta);
+    }
+#pragma unroll
+    for (int c = 0; c < S::NP; ++c) acc[n][c] = make_float2(0.f, 0.f);
+  }
+#pragma unroll 1
+  for (int k = 0; k < 7; ++k) {
+    const float* plane = fp + k * 49 * S::ST;
+    float wz[NT];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) wz[n] = es_kernel((float(k) - uz[n]) * sc2, a.beta);
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+      float2 row[NT][S::NP];  // sum over x of this footprint row
+#pragma unroll
+      for (int i = 0; i < 7; ++i) {
+        float2 v[(S::NP + 1) / 2 * 2];
+#pragma unroll
+        for (int c = 0; c < S::NP / 2; ++c) {
+          const float4 x = reinterpret_cast<const float4*>(plane + (j * 7 + i) * S::ST)[c];
+          v[2 * c] = make_float2(x.x, x.y);
+          v[2 * c + 1] = make_float2(x.z, x.w);
+        }
+        if constexpr (S::NP % 2) v[S::NP - 1] = reinterpret_cast<const float2*>(plane + (j * 7 + i) * S::ST)[S::NP - 1];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+#pragma unroll
+          for (int c = 0; c < S::NP; ++c)
+            row[n][c] = i ? __ffma2_rn(wx[n][i], v[c], row[n][c]) : __fmul2_rn(wx[n][0], v[c]);
+        }
+      }
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        const float w = wz[n] * wy[n][j];
+#pragma unroll
+        for (int c = 0; c < S::NP; ++c) acc[n][c] = __ffma2_rn(make_float2(w, w), row[n][c], acc[n][c]);
+      }
+    }
+  }
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+    if (t + 32 * n >= t1) continue;
+    const long long q = a.tidx[t + 32 * n];
+#pragma unroll
+    for (int c = 0; c < S::C; ++c) a.dst[c * a.nq + q] = c % 2 ? acc[n][c / 2].y : acc[n][c / 2].x;
+  }
+}
+template <int NM>
+__global__ void __launch_bounds__(kInterpBlock) k_interp7(InterpArgs<float> a) {
+  using S = Interp7<NM>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* fp = reinterpret_cast<float*>(smem_raw);  // [343][ST]
+  const int g = blockIdx.x, nf = a.nf;
+  const long long P = a.box.points();
+  const int4 g0 = a.tg0[g];
+  for (int p = threadIdx.x; p < 343; p += kInterpBlock) {
+    const int k = p / 49, r = p - k * 49, j = r / 7, i = r - j * 7;
+    int gx = g0.x + i, gy = g0.y + j, gz = g0.z + k;
+    gx -= gx >= nf ? nf : 0;
+    gy -= gy >= nf ? nf : 0;
+    gz -= gz >= nf ? nf : 0;
+    const float* src = a.F + box_at(a.box, gx, gy, gz);
+    float v[S::ST];
+#pragma unroll
+    for (int c = 0; c < S::ST; ++c) v[c] = c < S::C ? __ldg(src + c * P) : 0.f;
+#pragma unroll
+    for (int c = 0; c < S::ST / 4; ++c)
+      reinterpret_cast<float4*>(fp + p * S::ST)[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+  }
+  __syncthreads();
+  const int t1 = a.tgrp[g + 1], lane = threadIdx.x & 31;
+  for (int t = a.tgrp[g] + (threadIdx.x >> 5) * 64; t < t1; t += kInterpBlock / 32 * 64) {
+    if (t + 32 < t1) interp7_targets<NM, 2>(a, fp, t + lane, t1);
+    else interp7_targets<NM, 1>(a, fp, t + lane, t1);
+  }
+}
+
 template <typename T> struct ProjArgs {
-  const T* At;        // C x nq diffused values, sorted target order
-  const int* tidx;    // target -> field point
+  const T* At;        // C x nq diffused values
   T* A;               // field, C x nq (read: previous; written: projected)
   SurfStats* st;
   long long nq;
   T fb;
 };
 
+// Add a block's statistics to the step's: integer warp reductions (the bits of
+// non-negative doubles order like them; a butterfly of FP64 maxima in every warp
+// took a quarter of the projection), and a maximum that does not raise the
+// recorded one is not sent.
+template <typename T> __device__ __forceinline__ void surf_stats(const PointStats<T>& ps, SurfStats* st) {
+  __shared__ unsigned long long s_mx[kProjThreads / 32];
+  unsigned long long mx;
+  if constexpr (sizeof(T) == 4) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(ps.maxd));
+    mx = (unsigned long long)__double_as_longlong((double)__uint_as_float(m));
+  } else {
+    mx = warp_max_u64((unsigned long long)__double_as_longlong(ps.maxd));
+  }
+  const bool lead = (threadIdx.x & 31) == 0;
+  if (__any_sync(0xffffffffu, ps.flips | ps.nonfinite | ps.fallback)) {
+    const unsigned fl = __reduce_add_sync(0xffffffffu, (unsigned)ps.flips);
+    const unsigned nf = __reduce_add_sync(0xffffffffu, (unsigned)ps.nonfinite);
+    const unsigned fb = __reduce_add_sync(0xffffffffu, (unsigned)ps.fallback);
+    if (lead && fl) atomicAdd(&st->flips, (unsigned long long)fl);
+    if (lead && nf) atomicAdd(&st->nonfinite, (unsigned long long)nf);
+    if (lead && fb) atomicAdd(&st->fallback, (unsigned long long)fb);
+  }
+  if (lead) s_mx[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kProjThreads / 32; ++w) mx = s_mx[w] > mx ? s_mx[w] : mx;
+    if (mx > *reinterpret_cast<volatile unsigned long long*>(&st->maxd_bits)) atomicMax(&st->maxd_bits, mx);
+  }
+}
+
 // Projection of every target (Lemma 1.1) and the step statistics.
 template <typename T, int NM>
 __global__ void __launch_bounds__(kProjThreads) k_sproject(ProjArgs<T> a) {
   constexpr int C = NM * NM;
-  __shared__ double redd[32];
-  __shared__ int redi[32];
   const long long t = (long long)blockIdx.x * kProjThreads + threadIdx.x;
   PointStats<T> ps;
   if (t < a.nq) {
-    const long long q = a.tidx[t];
     T m[C], old[C], bb[C], sg;
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       m[c] = a.At[c * a.nq + t];
-      old[c] = a.A[c * a.nq + q];
+      old[c] = a.A[c * a.nq + t];
     }
     bool fin = true;
 #pragma unroll
@@ -368,21 +669,12 @@ __global__ void __launch_bounds__(kProjThreads) k_sproject(ProjArgs<T> a) {
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       d = fmax(d, fabs(bb[c] - old[c]));
-      a.A[c * a.nq + q] = bb[c];
+      a.A[c * a.nq + t] = bb[c];
     }
     ps.maxd = d;
     ps.flips = (det_sign<NM>(old) != sg) ? 1 : 0;
   }
-  const double mx = block_max((double)ps.maxd, redd);
-  const int fl = block_sum(ps.flips, redi);
-  const int nfin = block_sum(ps.nonfinite, redi);
-  const int nfb = block_sum(ps.fallback, redi);
-  if (threadIdx.x == 0) {
-    atomicMax(&a.st->maxd_bits, (unsigned long long)__double_as_longlong(mx));
-    if (fl) atomicAdd(&a.st->flips, (unsigned long long)fl);
-    if (nfin) atomicAdd(&a.st->nonfinite, (unsigned long long)nfin);
-    if (nfb) atomicAdd(&a.st->fallback, (unsigned long long)nfb);
-  }
+  surf_stats(ps, a.st);
 }
 
 // Step statistics of the volume-preserving step: compare the previous field
@@ -390,8 +682,6 @@ __global__ void __launch_bounds__(kProjThreads) k_sproject(ProjArgs<T> a) {
 template <typename T, int NM>
 __global__ void __launch_bounds__(kProjThreads) k_sdelta(const T* old, const T* A, long long nq, SurfStats* st) {
   constexpr int C = NM * NM;
-  __shared__ double redd[32];
-  __shared__ int redi[32];
   const long long q = (long long)blockIdx.x * kProjThreads + threadIdx.x;
   PointStats<T> ps;
   if (q < nq) {
@@ -409,14 +699,7 @@ __global__ void __launch_bounds__(kProjThreads) k_sdelta(const T* old, const T* 
     ps.nonfinite = fin ? 0 : 1;
     ps.flips = (det_sign<NM>(o) != det_sign<NM>(b)) ? 1 : 0;
   }
-  const double mx = block_max((double)ps.maxd, redd);
-  const int fl = block_sum(ps.flips, redi);
-  const int nfin = block_sum(ps.nonfinite, redi);
-  if (threadIdx.x == 0) {
-    atomicMax(&st->maxd_bits, (unsigned long long)__double_as_longlong(mx));
-    if (fl) atomicAdd(&st->flips, (unsigned long long)fl);
-    if (nfin) atomicAdd(&st->nonfinite, (unsigned long long)nfin);
-  }
+  surf_stats(ps, st);
 }
 
 // Weighted selection of Algorithm 3 (Sec. 7 on surfaces): with points ordered
@@ -696,9 +979,11 @@ struct mbo_surface_ctx {
   int tgroups = 0;   // target groups
   int cg = 1, chgroups = 1;  // channels per spreading block, channel groups
   size_t tile_bytes = 0;
-  mbo_handle fine = nullptr;  // 3-D FFT diffusion on the nf^3 grid
-  void* F = nullptr;          // grid, C x nf^3
-  void* At = nullptr;         // diffused values in sorted target order, C x nq
+  GridBox box{};              // FP32: the box of all footprints; FP64: the whole grid
+  BoxDiffusion bd{};          // FP32: diffusion between points of the box
+  mbo_handle fine = nullptr;  // FP64: 3-D FFT diffusion on the nf^3 grid
+  void* F = nullptr;          // grid values of the box, C channels
+  void* At = nullptr;         // diffused values, C x nq
   // volume-preserving step (allocated on first use)
   void* Au = nullptr;                      // diffused values in the caller's order, C x nq
   unsigned long long* vkeys = nullptr;     // one selection key per point
@@ -711,6 +996,9 @@ struct mbo_surface_ctx {
   int* sidx = nullptr;
   int* gsrc = nullptr;
   int* gt0 = nullptr;
+  int4* sg0 = nullptr;        // FP32, width 7: source group -> footprint start on the grid
+  int* seg = nullptr;         // FP32, width 7: segment -> first group
+  int nseg = 0;
   int* bgrp = nullptr;
   int* bid = nullptr;
   void* tu = nullptr;         // V4<T> targets
@@ -788,7 +1076,13 @@ int spread_cg(int C, size_t elem, size_t tv, size_t limit) {
 
 template <typename T, int CG> cudaError_t spread_run(const SpreadArgs<T>& a, dim3 grid, size_t smem,
                                                      cudaStream_t st) {
-  auto k = a.W == 7 ? k_spread<T, CG, 7> : k_spread<T, CG, 0>;
+  if constexpr (sizeof(T) == 4) {
+    if (a.W == 7) {
+      k_spread7<CG><<<dim3(a.nseg, grid.y), kSpread7Threads, 0, st>>>(a);
+      return cudaGetLastError();
+    }
+  }
+  auto k = sizeof(T) == 8 && a.W == 7 ? k_spread<T, CG, sizeof(T) == 8 ? 7 : 0> : k_spread<T, CG, 0>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -805,8 +1099,12 @@ template <typename T> cudaError_t launch_spread(mbo_surface_ctx* s, const void* 
   a.gsrc = s->gsrc;
   a.gt0 = s->gt0;
   a.bgrp = s->bgrp;
+  a.g0 = s->sg0;
+  a.seg = s->seg;
+  a.nseg = s->nseg;
   a.bid = s->bid;
   a.F = static_cast<T*>(s->F);
+  a.box = s->box;
   a.nq = s->nq;
   a.C = s->C;
   a.nf = s->prm.nf;
@@ -829,7 +1127,13 @@ template <typename T> cudaError_t launch_spread(mbo_surface_ctx* s, const void* 
 
 template <typename T, int NM> cudaError_t interp_run(const InterpArgs<T>& a, int groups, size_t smem,
                                                       cudaStream_t st) {
-  auto k = a.W == 7 ? k_interp<T, NM, 7> : k_interp<T, NM, 0>;
+  if constexpr (sizeof(T) == 4 && (NM == 2 || NM == 3)) {
+    if (a.W == 7) {
+      k_interp7<NM><<<groups, kInterpBlock, 343 * Interp7<NM>::ST * sizeof(float), st>>>(a);
+      return cudaGetLastError();
+    }
+  }
+  auto k = a.W == 7 ? k_interp<T, NM, sizeof(T) == 4 && (NM == 2 || NM == 3) ? 0 : 7> : k_interp<T, NM, 0>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -838,9 +1142,10 @@ template <typename T, int NM> cudaError_t interp_run(const InterpArgs<T>& a, int
   return cudaGetLastError();
 }
 
-template <typename T> cudaError_t launch_interp(mbo_surface_ctx* s, void* dst, bool scatter, cudaStream_t st) {
+template <typename T> cudaError_t launch_interp(mbo_surface_ctx* s, void* dst, cudaStream_t st) {
   InterpArgs<T> a;
   a.F = static_cast<const T*>(s->F);
+  a.box = s->box;
   a.tu = static_cast<const V4<T>*>(s->tu);
   a.tidx = s->tidx;
   a.tgrp = s->tgrp;
@@ -849,7 +1154,6 @@ template <typename T> cudaError_t launch_interp(mbo_surface_ctx* s, void* dst, b
   a.nq = s->nq;
   a.nf = s->prm.nf;
   a.W = s->prm.width;
-  a.scatter = scatter;
   a.beta = (T)s->prm.beta;
   const int W3 = s->prm.width * s->prm.width * s->prm.width;
   const int CP = s->C == 1 ? 1 : (sizeof(T) == 4 ? (s->C + 3) / 4 * 4 : (s->C + 1) / 2 * 2);
@@ -865,7 +1169,6 @@ template <typename T> cudaError_t launch_interp(mbo_surface_ctx* s, void* dst, b
 template <typename T> cudaError_t launch_project(mbo_surface_ctx* s, void* A, cudaStream_t st) {
   ProjArgs<T> a;
   a.At = static_cast<const T*>(s->At);
-  a.tidx = s->tidx;
   a.A = static_cast<T*>(A);
   a.st = s->st;
   a.nq = s->nq;
@@ -880,22 +1183,24 @@ template <typename T> cudaError_t launch_project(mbo_surface_ctx* s, void* A, cu
   return cudaGetLastError();
 }
 
-mbo_status surface_diffusion(mbo_surface_ctx* s, const void* A, void* dst, bool scatter, cudaStream_t st) {
-  const long long P = (long long)s->prm.nf * s->prm.nf * s->prm.nf;
+mbo_status surface_diffusion(mbo_surface_ctx* s, const void* A, void* dst, cudaStream_t st) {
   const size_t elem = s->dtype == MBO_F32 ? 4 : 8;
-  SCK(cudaMemsetAsync(s->F, 0, (size_t)s->C * P * elem, st));
+  SCK(cudaMemsetAsync(s->F, 0, (size_t)s->C * s->box.points() * elem, st));
   SCK(timed(s, 0, st, [&] {
     return s->dtype == MBO_F32 ? launch_spread<float>(s, A, st) : launch_spread<double>(s, A, st);
   }));
-  mbo_status rc = MBO_OK;
-  timed(s, 1, st, [&] {
-    rc = mbo_diffuse(s->fine, s->F, s->F, st);
-    return cudaSuccess;
-  });
-  if (rc != MBO_OK) return sfail(s, rc, "grid diffusion: %s", mbo_last_error(s->fine));
+  if (s->dtype == MBO_F32) {
+    SCK(timed(s, 1, st, [&] { return box_diffuse(s->bd, static_cast<float*>(s->F), st); }));
+  } else {
+    mbo_status rc = MBO_OK;
+    timed(s, 1, st, [&] {
+      rc = mbo_diffuse(s->fine, s->F, s->F, st);
+      return cudaSuccess;
+    });
+    if (rc != MBO_OK) return sfail(s, rc, "grid diffusion: %s", mbo_last_error(s->fine));
+  }
   SCK(timed(s, 2, st, [&] {
-    return s->dtype == MBO_F32 ? launch_interp<float>(s, dst, scatter, st)
-                               : launch_interp<double>(s, dst, scatter, st);
+    return s->dtype == MBO_F32 ? launch_interp<float>(s, dst, st) : launch_interp<double>(s, dst, st);
   }));
   return MBO_OK;
 }
@@ -980,7 +1285,7 @@ mbo_status mbo_surface_destroy(mbo_surface s) {
   else prev = -1;
   cudaDeviceSynchronize();
   if (s->fine) mbo_destroy(s->fine);
-  void* bufs[] = {s->F, s->At, s->su, s->sidx, s->gsrc, s->gt0, s->bgrp, s->bid,
+  void* bufs[] = {s->bd.tabs, s->bd.W1, s->bd.W2, s->F, s->At, s->su, s->sidx, s->gsrc, s->gt0, s->bgrp, s->bid, s->sg0, s->seg,
                   s->tu, s->tidx, s->tgrp, s->tg0, s->st, s->Au, s->vkeys, s->vss, s->vws, s->vw};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -1056,10 +1361,19 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
       u[a] = std::min(std::max(v, 0.0), std::nextafter((double)nf, 0.0));
     }
   };
-  // sources: key (bin, footprint start in the bin tile); targets: footprint start
+  // sources: key (bin, footprint start in the bin tile), or for k_spread7 the
+  // footprint start on the grid, z fastest; targets: footprint start
+  const bool columns = dtype == MBO_F32 && W == 7;
+  std::vector<char> bin_used((size_t)nb * nb * nb, 0);
   std::vector<long long> skey(nq), tkey(nq);
   std::vector<V4<double>> sd(nq), td(nq);
-  std::vector<int> sgx(3 * nq);
+  // extent of all footprints (unwrapped): sources cover W + 1 points from an
+  // even start in x and y, everything else W
+  int ext_lo[3] = {nf, nf, nf}, ext_hi[3] = {-nf, -nf, -nf};
+  auto cover = [&](int a, int from, int count) {
+    ext_lo[a] = std::min(ext_lo[a], from);
+    ext_hi[a] = std::max(ext_hi[a], from + count);
+  };
   for (int64_t i = 0; i < nq; ++i) {
     double u[3];
     int b[3], t0[3], g[3];
@@ -1072,12 +1386,22 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
       t0[a] = std::min(std::max(t0[a], 0), kBin);
       if (a < 2) t0[a] &= ~1;
       g[a] = b[a] * kBin - W / 2 + t0[a];
+      if (columns) {
+        g[a] = (int)std::ceil(u[a] - 0.5 * W);
+        if (a < 2) g[a] -= g[a] & 1;
+      }
+      cover(a, g[a], a < 2 ? W + 1 : W);
     }
     const long long bin = ((long long)b[2] * nb + b[1]) * nb + b[0];
-    skey[i] = bin * 4096 + (t0[2] << 8 | t0[1] << 4 | t0[0]);
+    bin_used[bin] = 1;
+    skey[i] = columns ? (((long long)(g[1] + kMaxW) << 12 | (g[0] + kMaxW)) << 12 | (g[2] + kMaxW))
+                      : bin * 4096 + (t0[2] << 8 | t0[1] << 4 | t0[0]);
     sd[i] = V4<double>{u[0] - g[0], u[1] - g[1], u[2] - g[2], wq[i]};
     grid_coord(xc + 3 * i, u);
-    for (int a = 0; a < 3; ++a) g[a] = (int)std::ceil(u[a] - 0.5 * W);
+    for (int a = 0; a < 3; ++a) {
+      g[a] = (int)std::ceil(u[a] - 0.5 * W);
+      cover(a, g[a], W);
+    }
     // wrapped start on the periodic grid (u >= 0, so g >= -W/2)
     const int gx = (g[0] + nf) % nf, gy = (g[1] + nf) % nf, gz = (g[2] + nf) % nf;
     tkey[i] = ((long long)gz * nf + gy) * nf + gx;
@@ -1088,7 +1412,8 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
   std::iota(tperm.begin(), tperm.end(), 0);
   std::stable_sort(sperm.begin(), sperm.end(), [&](int x, int y) { return skey[x] < skey[y]; });
   std::stable_sort(tperm.begin(), tperm.end(), [&](int x, int y) { return tkey[x] < tkey[y]; });
-  std::vector<int> gsrc, gt0, bgrp, bid, tgrp;
+  std::vector<int> gsrc, gt0, bgrp, bid, tgrp, seg;
+  std::vector<int4> sg0;
   std::vector<int4> tg0;
   std::vector<V4<double>> sds(nq), tds(nq);
   for (int64_t r = 0; r < nq; ++r) {
@@ -1096,7 +1421,10 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
     sds[r] = sd[i];
     if (r == 0 || skey[i] != skey[sperm[r - 1]]) {
       const long long bin = skey[i] / 4096;
-      if (r == 0 || bin != skey[sperm[r - 1]] / 4096) {
+      if (columns) {
+        sg0.push_back(make_int4((int)(skey[i] >> 12 & 4095) - kMaxW, (int)(skey[i] >> 24) - kMaxW,
+                                (int)(skey[i] & 4095) - kMaxW, 0));
+      } else if (r == 0 || bin != skey[sperm[r - 1]] / 4096) {
         bid.push_back((int)bin);
         bgrp.push_back((int)gsrc.size());
       }
@@ -1114,10 +1442,19 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
   gsrc.push_back((int)nq);
   tgrp.push_back((int)nq);
   bgrp.push_back((int)gt0.size());
+  // segments: runs of a column's groups, up to kSegSources sources where a group
+  // does not hold more, without gaps of a whole footprint in z
+  for (size_t g = 0; g < sg0.size(); ++g) {
+    const bool run = g > 0 && sg0[g].x == sg0[g - 1].x && sg0[g].y == sg0[g - 1].y &&
+                     sg0[g].z - sg0[g - 1].z < W && gsrc[g + 1] - gsrc[seg.back()] <= kSegSources;
+    if (!run) seg.push_back((int)g);
+  }
+  s->nseg = (int)seg.size();
+  seg.push_back((int)sg0.size());
   s->nbins = (int)bid.size();
-  s->sgroups = (int)gt0.size();
+  s->sgroups = (int)gsrc.size() - 1;
   s->tgroups = (int)tg0.size();
-  prm.bins = s->nbins;
+  prm.bins = std::count(bin_used.begin(), bin_used.end(), 1);
 
   // channel groups of the spreading tile
   const size_t elem = dtype == MBO_F32 ? 4 : 8;
@@ -1133,12 +1470,21 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
   }
 
   // the grid's FFT diffusion with the deconvolved heat factor
-  const int64_t dims[3] = {nf, nf, nf};
-  mbo_status rc = mbo_create(&s->fine, 3, dims, n, 1.0, dtype, nullptr);
-  if (rc != MBO_OK) {
-    snprintf(s->err, sizeof(s->err), "grid plan: %s", mbo_status_string(rc));
-    mbo_surface_destroy(s);
-    return rc;
+  mbo_status rc = MBO_OK;
+  for (int a = 0; a < 3; ++a) {
+    // an axis whose footprints wrap keeps all of it
+    const bool inside = dtype == MBO_F32 && ext_lo[a] >= 0 && ext_hi[a] <= nf;
+    s->box.b0[a] = inside ? ext_lo[a] : 0;
+    s->box.bn[a] = inside ? ext_hi[a] - ext_lo[a] : nf;
+  }
+  if (dtype == MBO_F64) {
+    const int64_t dims[3] = {nf, nf, nf};
+    rc = mbo_create(&s->fine, 3, dims, n, 1.0, dtype, nullptr);
+    if (rc != MBO_OK) {
+      snprintf(s->err, sizeof(s->err), "grid plan: %s", mbo_status_string(rc));
+      mbo_surface_destroy(s);
+      return rc;
+    }
   }
   std::vector<double> gx, gwt, mult(nf);
   gauss_legendre(128, gx, gwt);
@@ -1160,14 +1506,22 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
     mult[k] = nf * (prm.h / (2.0 * M_PI)) * win * std::exp(-(double)kf * kf * prm.h * prm.h * tau) / (psi * psi);
   }
   const double* mm[3] = {mult.data(), mult.data(), mult.data()};
-  if (!set_axis_multipliers(s->fine, mm)) {
+  if (dtype == MBO_F64 && !set_axis_multipliers(s->fine, mm)) {
     snprintf(s->err, sizeof(s->err), "grid multipliers: %s", cudaGetErrorString(cudaGetLastError()));
     mbo_surface_destroy(s);
     return MBO_ERR_CUDA;
   }
+  if (dtype == MBO_F32) {
+    rc = box_create(s->bd, s->box, nf, n, prm.M, mult.data(), maxsm, s->bytes);
+    if (rc != MBO_OK) {
+      snprintf(s->err, sizeof(s->err), "grid plan: %s", mbo_status_string(rc));
+      mbo_surface_destroy(s);
+      return rc;
+    }
+  }
 
   // device tables
-  const long long P = (long long)nf * nf * nf;
+  const long long P = s->box.points();
   auto alloc = [&](void** p, size_t b) {
     if (cudaMalloc(p, std::max<size_t>(b, 16)) != cudaSuccess) return false;
     s->bytes += b;
@@ -1177,6 +1531,7 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
   if (!alloc(&s->F, (size_t)s->C * P * elem) || !alloc(&s->At, (size_t)s->C * nq * elem) ||
       !alloc(&s->su, nq * v4) || !alloc((void**)&s->sidx, nq * sizeof(int)) ||
       !alloc((void**)&s->gsrc, gsrc.size() * sizeof(int)) || !alloc((void**)&s->gt0, gt0.size() * sizeof(int)) ||
+      !alloc((void**)&s->sg0, sg0.size() * sizeof(int4)) || !alloc((void**)&s->seg, seg.size() * sizeof(int)) ||
       !alloc((void**)&s->bgrp, bgrp.size() * sizeof(int)) || !alloc((void**)&s->bid, bid.size() * sizeof(int)) ||
       !alloc(&s->tu, nq * v4) || !alloc((void**)&s->tidx, nq * sizeof(int)) ||
       !alloc((void**)&s->tgrp, tgrp.size() * sizeof(int)) || !alloc((void**)&s->tg0, tg0.size() * sizeof(int4)) ||
@@ -1196,6 +1551,8 @@ mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq, co
   cudaMemcpy(s->gsrc, gsrc.data(), gsrc.size() * sizeof(int), cudaMemcpyHostToDevice);
   cudaMemcpy(s->gt0, gt0.data(), gt0.size() * sizeof(int), cudaMemcpyHostToDevice);
   cudaMemcpy(s->bgrp, bgrp.data(), bgrp.size() * sizeof(int), cudaMemcpyHostToDevice);
+  cudaMemcpy(s->sg0, sg0.data(), sg0.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  cudaMemcpy(s->seg, seg.data(), seg.size() * sizeof(int), cudaMemcpyHostToDevice);
   cudaMemcpy(s->bid, bid.data(), bid.size() * sizeof(int), cudaMemcpyHostToDevice);
   cudaMemcpy(s->tidx, tperm.data(), nq * sizeof(int), cudaMemcpyHostToDevice);
   cudaMemcpy(s->tgrp, tgrp.data(), tgrp.size() * sizeof(int), cudaMemcpyHostToDevice);
@@ -1218,13 +1575,13 @@ mbo_status mbo_surface_get_params(mbo_surface s, mbo_surface_params* p) {
 
 mbo_status mbo_surface_diffuse(mbo_surface s, const void* A, void* A_tilde, void* stream) {
   if (!s || !A || !A_tilde || ((uintptr_t)A & 15) || ((uintptr_t)A_tilde & 15)) return MBO_ERR_INVALID_ARG;
-  return surface_diffusion(s, A, A_tilde, true, static_cast<cudaStream_t>(stream));
+  return surface_diffusion(s, A, A_tilde, static_cast<cudaStream_t>(stream));
 }
 
 mbo_status mbo_surface_step(mbo_surface s, void* A, mbo_stats* stats, void* stream) {
   if (!s || !A || ((uintptr_t)A & 15)) return MBO_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  mbo_status rc = surface_diffusion(s, A, s->At, false, st);
+  mbo_status rc = surface_diffusion(s, A, s->At, st);
   if (rc != MBO_OK) return rc;
   SCK(cudaMemsetAsync(s->st, 0, sizeof(SurfStats), st));
   SCK(timed(s, 3, st, [&] {
@@ -1292,7 +1649,7 @@ mbo_status mbo_surface_step_volume(mbo_surface s, void* A, double volume, mbo_st
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the diffused field in the caller's order; the previous field kept for the statistics
-  mbo_status rc = surface_diffusion(s, A, s->Au, true, st);
+  mbo_status rc = surface_diffusion(s, A, s->Au, st);
   if (rc != MBO_OK) return rc;
   SCK(cudaMemcpyAsync(s->At, A, fbytes, cudaMemcpyDeviceToDevice, st));
   // dE keys (the flat-torus volume step's kernels, on the nq points), the
