@@ -38,6 +38,10 @@ inline __host__ __device__ constexpr int wrow_minb(int N, int NM) {
              ? (4 * (16384 / (32 * (NM <= 3 ? 96 : 128)))) / (wrow_threads(N, NM) / 32)
              : 1;
 }
+// Helper factor of the x pass on small grids (k_wrow's HX): up to 256 - 320 threads.
+inline __host__ __device__ constexpr int wrow_helpers(int N, int NM) {
+  return w_r(N) > 1 || NM > 3 ? 1 : wrow_threads(N, NM) <= 64 ? 4 : 2;
+}
 inline __host__ __device__ constexpr int wcol_minb(int L, int TX) {
   return 512 / (TX * w_r(L) * w_lq(L)) > 0 ? 512 / (TX * w_r(L) * w_lq(L)) : 1;
 }
