@@ -757,7 +757,16 @@ __device__ __forceinline__ R polar_newton(const R* m, R* b, R& est, R skip_below
 // finish.  est and the routing of small or singular points are as in
 // polar_newton (points not iterated at all return done = true with est <=
 // skip_below).  The returned class is the sign of det of the last iterate.
+// Inside a phase the diffused matrix is close to a multiple of an orthogonal
+// one, and the first scaled step already lands next to the polar factor.  After
+// a Newton step every singular value is at least 1 ((s + 1/s) / 2), so |X|_F^2 - 3
+// bounds each s^2 - 1: below kPolarNear the next unscaled step ends within
+// (2e-4)^2 / 2 = 2e-8 of orthogonality, under the rounding of the iterate, and
+// the other two steps are left out (about 110 of the projection's 250
+// instructions; two-phase 1536 x 2048, n = 3: step 313 -> 303 us; smooth 256^3 with
+// isolated reflections: 1175 -> 1117 us).
 constexpr float kPolarAccept = 3e-4f;
+constexpr float kPolarNear = 4e-4f;
 
 __device__ __forceinline__ float polar3_fixed(const float* m, float* b, float& est, float skip_below,
                                               float cof2_floor, bool& done) {
@@ -787,10 +796,15 @@ __device__ __forceinline__ float polar3_fixed(const float* m, float* b, float& e
       nx = 0.f;
       nc = 0.f;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        nx += X[k] * X[k];
-        nc += C[k] * C[k];
+      for (int k = 0; k < 9; ++k) nx += X[k] * X[k];
+      if (nx - 3.f <= kPolarNear) {  // one unscaled step is all that is left
+        const float c = 0.5f * __frcp_rn(det);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) b[k] = 0.5f * X[k] + c * C[k];
+        return det >= 0.f ? 1.f : -1.f;
       }
+#pragma unroll
+      for (int k = 0; k < 9; ++k) nc += C[k] * C[k];
     }
     const float zf = rsqrtf(rsqrtf(__fdividef(nc, det * det * nx)));
     const float a = 0.5f * zf;
