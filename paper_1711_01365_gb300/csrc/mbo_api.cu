@@ -52,47 +52,57 @@ FastDiv make_div(unsigned d) {
   return f;
 }
 
-// Radix plan of N = 2^a 3^b: as few stages of radix 16, 12, 9, 8, 6, 4, 3 or 2
-// as possible, and among those plans the one of least butterfly work (operations
-// per point of a length-r DFT, by how the registers compute it).  The stages
-// with the most factors of two come first, so that the spans below them stay
-// multiples of 8 (affine addressing) as long as possible.  Stage twiddle
-// offsets are assigned in stage order.
-struct RadixCost { int r, a, b; double ops; };
-// (small_code: without 16 and 12)
-const RadixCost kRadix[] = {{16, 4, 0, 10.5}, {12, 2, 1, 9.3}, {9, 0, 2, 10.2}, {8, 3, 0, 7.0},
-                            {6, 1, 1, 7.3},   {4, 2, 0, 4.0},  {3, 0, 1, 5.3},  {2, 1, 0, 2.0}};
+// Radix plan of N = 2^a 3^b in stages of radix 16, 12, 9, 8, 6, 4, 3 and 2.  Large
+// fields: as few stages as possible, and among those plans the one of least
+// butterfly work (486 = 6 9 9 and 648 = 8 9 9 instead of six and five stages with
+// one per factor of three: the 486 x 648, n = 3 step 80.1 -> 58.4 us).  Small
+// fields: the least time for one block, whose chain of stages and whose first
+// fetch of every butterfly's instructions (about 4 KB/us per SM) both count:
+// equal radices share their code.  The stages with the most factors of two come
+// first, so that the spans below them stay multiples of 8 (affine addressing) as
+// long as possible.  Stage twiddle offsets are assigned in stage order.
+struct RadixCost {
+  int r, a, b;
+  double ops;           // operations per point of a length-r DFT
+  // KB of instructions of the FP32 butterflies (both directions) and the
+  // fixed-point one (radix 2 above its size: 128 = 8 8 2 measured slower than 8 4 4)
+  double kb32, kb64;
+};
+const RadixCost kRadix[] = {{16, 4, 0, 10.5, 13, 45}, {12, 2, 1, 9.3, 10, 30}, {9, 0, 2, 10.2, 8, 13},
+                            {8, 3, 0, 7.0, 5, 8},     {6, 1, 1, 7.3, 3.6, 3.5}, {4, 2, 0, 4.0, 2, 3.5},
+                            {3, 0, 1, 5.3, 1.4, 2},   {2, 1, 0, 2.0, 2.5, 4}};
 
-// from: first entry of kRadix to try
-void search_plan(int a, int b, int from, int depth, int* cur, double ops, int& best_n, double& best_ops,
-                 int* best) {
+void search_plan(PlanFor want, int a, int b, int from, int depth, int* cur, double cost, int& best_n,
+                 double& best, int* rad) {
   if (a == 0 && b == 0) {
-    if (depth < best_n || (depth == best_n && ops < best_ops)) {
+    if (cost < best) {
       best_n = depth;
-      best_ops = ops;
-      std::copy(cur, cur + depth, best);
+      best = cost;
+      std::copy(cur, cur + depth, rad);
     }
     return;
   }
-  if (depth >= best_n || depth >= kMaxStages) return;
+  if (depth >= kMaxStages) return;
   for (int i = from; i < 8; ++i) {
     const RadixCost& r = kRadix[i];
     if (r.a > a || r.b > b) continue;
     cur[depth] = r.r;
-    search_plan(a - r.a, b - r.b, i, depth + 1, cur, ops + r.ops, best_n, best_ops, best);
+    const bool fresh = depth == 0 || cur[depth - 1] != r.r;  // radices descend: equal ones are neighbours
+    const double code = fresh ? (want == PlanFor::kSmall32 ? r.kb32 : r.kb64) / 4.0 : 0.0;  // us
+    const double step = want == PlanFor::kThroughput ? 1000.0 + r.ops : 2.0 + code;          // two stages of 1 us
+    search_plan(want, a - r.a, b - r.b, i, depth + 1, cur, cost + step, best_n, best, rad);
   }
 }
 
-Plan make_plan(int N, bool small_code) {
+Plan make_plan(int N, PlanFor want) {
   Plan p{};
   p.len = N;
   int a, b;
   factor23(N, a, b);
   int rad[kMaxStages], cur[kMaxStages];
-  int ns = kMaxStages + 1;
-  double ops = 0.0;
-  search_plan(a, b, small_code ? 2 : 0, 0, cur, 0.0, ns, ops, rad);
-  // 2^10 and 2^11 need four radix-8 stages: always within kMaxStages
+  int ns = 0;
+  double cost = 1e300;
+  search_plan(want, a, b, 0, 0, cur, 0.0, ns, cost, rad);
   std::stable_sort(rad, rad + ns, [](int x, int y) {
     auto twos = [](int v) { int t = 0; while (v % 2 == 0) { v /= 2; ++t; } return t; };
     return twos(x) > twos(y);
@@ -116,7 +126,9 @@ Plan make_plan(int N, bool small_code) {
   return p;
 }
 
-constexpr long long kSmallCode = 1500000;
+// Elements up to which a field's network passes are planned for one block's
+// time.  FP64: 128^2, n = 2: y pass 29 -> 23 us, x pass 31 -> 23 us.
+constexpr long long kSmall64 = 1500000, kSmall32 = 300000;
 
 Plan axis_plan(const Geom& g, int axis, bool f32) {
   const int N = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
@@ -128,12 +140,8 @@ Plan axis_plan(const Geom& g, int axis, bool f32) {
     p.lq = N / p.rad0 == 1024 ? 32 : 16;
     return p;
   }
-  // FP64 (fixed point): the butterflies of radix 16 and 12 are 45 and 30 KB of
-  // instructions, which every SM fetches once per pass at about 4 KB/us (ncu:
-  // warps wait for instructions first of all); up to kSmallCode elements that
-  // costs more than the stage they save (128^2, n = 2: y pass 29 -> 23 us, x pass
-  // 31 -> 23 us)
-  return make_plan(N, !f32 && g.P * g.Q <= kSmallCode);
+  if (g.P * g.Q > (f32 ? kSmall32 : kSmall64)) return make_plan(N);
+  return make_plan(N, f32 ? PlanFor::kSmall32 : PlanFor::kSmall64);
 }
 
 int plan_twiddles(const Plan& p) {
@@ -846,16 +854,28 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
   cudaGetDevice(&h->dev);
   // launch shapes
   h->tx = pick_tx(g.nx, dtype == MBO_F32 ? 8 : 4);
-  // measured on GB300 (1024^2, n = 3): 192 threads best for FP32 and FP64 rows.
-  // FP64 (168 registers: 384 threads fit on an SM): 192 from 256 points on (two
-  // blocks per SM at 1024, one round of butterflies at 256 - 648), 384 where a row
-  // fills the SM's shared memory, 128 for short rows (128^2, n = 2: 64 threads 26.6
-  // us, 128 threads 23.1 us)
+  // Threads of the network passes, measured on GB300.  FP32 rows: a thread per
+  // point of a short row (162 points, n = 3: 64 threads 22.9 us, 192 threads 18.7;
+  // 96^3, n = 2: 64 threads 48.5 us, 96 threads 44.5, 128 threads 53.3), then 192
+  // (486 x 648, n = 3: 128 threads 38.3 us, 192 threads 34.5, 256 threads 39.3), 256
+  // for long rows of several planes (1296 points, n = 3: 192 threads 110 us, 256
+  // threads 103).  FP64 rows (168 registers: 384 threads fit on an SM): 192 from
+  // 256 points on, 384 where a row fills the SM's shared memory, 128 for short
+  // rows (128^2, n = 2: 64 threads 26.6 us, 128 threads 23.1 us).
   if (dtype == MBO_F32)
-    h->row_threads = g.nx >= 2048 ? 256 : g.nx >= 1024 ? 192 : (g.nx >= 256 ? 128 : (g.nx >= 64 ? 64 : 32));
+    h->row_threads = g.nx <= 192 ? std::max(32, (g.nx + 31) / 32 * 32) : g.nx >= 1200 && n >= 3 ? 256 : 192;
   else
     h->row_threads = row_smem_bytes(g, 8, false) > 114 * 1024 ? 384 : g.nx >= 256 ? 192 : g.nx >= 64 ? 128 : 32;
-  h->axis_threads = dtype == MBO_F32 ? 256 : 128;  // FP64: 168 registers, three blocks per SM
+  // Strided passes: as many threads as a stage of the longest network axis has
+  // butterflies (tiles of 96 x 8, n = 3, 96^3: 256 threads 78 us, 64 threads 37.5;
+  // 486 x 8: 64 threads 31.1 us, 256 threads 23.3), 256 at most in FP32 and 128 in
+  // FP64 (168 registers, three blocks per SM: 1024^2, n = 3: 256 threads 480 us,
+  // 128 threads 338).
+  int longest = 0;
+  for (int ax = 1; ax < ndim; ++ax)
+    if (!axis_plan(g, ax, dtype == MBO_F32).lq) longest = std::max(longest, ax == 1 ? g.ny : g.nz);
+  if (dtype == MBO_F32) h->axis_threads = longest <= 96 ? 64 : longest <= 192 ? 128 : longest <= 288 ? 192 : 256;
+  else h->axis_threads = longest <= 96 ? 64 : 128;
   if (dtype == MBO_F32) {
     // FP32 warp-plan strided passes, measured on GB300: 16-column tiles (one
     // 128-byte line per tile row) where an axis of 512 is strided (512^3:

@@ -239,7 +239,8 @@ inline mbo_status box_create(BoxDiffusion& b, const GridBox& box, int nf, int n,
   b.xlast = (b.C & 1) && b.na == 2 * M + 1 ? M + 1 : b.na;
   b.plan = make_plan(nf);
   b.inv_p = (float)(1.0 / ((double)nf * nf * nf));
-  b.row_threads = nf >= 1024 ? 256 : nf >= 256 ? 128 : 64;
+  // a thread per butterfly of a radix-12 stage
+  b.row_threads = std::max(64, std::min(256, (b.Q * nf / 12 + 31) / 32 * 32));
   if ((size_t)b.Q * row_pad(nf) * sizeof(float2) > (size_t)maxsm ||
       (size_t)row_pad(nf) * kBoxTx * sizeof(float2) > (size_t)maxsm)
     return MBO_ERR_UNSUPPORTED_SIZE;

@@ -224,8 +224,10 @@ cudaError_t launch_project(const Geom& g, const R* At, R* B, int8_t* det_sign,
 // Plan helpers (mbo_api.cu).
 bool factor23(int64_t N, int& a, int& b);
 FastDiv make_div(unsigned d);
-// small_code: radices up to 9 only
-Plan make_plan(int N, bool small_code = false);
+// What a network plan is chosen for: throughput, or the time of one block in an
+// FP32 or a fixed-point pass.
+enum class PlanFor { kThroughput, kSmall32, kSmall64 };
+Plan make_plan(int N, PlanFor want = PlanFor::kThroughput);
 // Plan of one axis of a geometry: the warp-cooperative plan (FP32, lengths
 // 256, 512, 768, 1024, 1536, 2048; strided axes need nx % 4 == 0) where one
 // exists, else make_plan.
