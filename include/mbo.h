@@ -116,7 +116,9 @@ MBO_API void mbo_default_config(mbo_config* cfg);
 
 /* The launch shapes a handle uses (after any autotuning): row_threads,
  * axis_threads, axis_tx, axis_stages and pdl (1 on, 2 off) filled in; the
- * other fields as the handle was created with. */
+ * other fields as the handle was created with.  (Where axis_tx was automatic,
+ * axes without a warp plan may take tiles of another width than it reports:
+ * full ones with a ragged last tile, or narrower ones for small fields.) */
 MBO_API mbo_status mbo_launch_config(mbo_handle h, mbo_config* out);
 
 /* Create a handle for one field geometry.

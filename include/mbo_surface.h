@@ -93,9 +93,10 @@ MBO_API mbo_status mbo_surface_peanut_band(double dx, double wb, int p, double* 
  *             spreading error is then about 10^(1 - width): below 1e-7 the
  *             non-uniform transforms, not eps, set the accuracy).
  * The oversampled grid has nf = the smallest 2^a 3^b >= max(4M, 2 width, 8)
- * points per axis (MBO_ERR_UNSUPPORTED_SIZE above 2048).  Allocates that
- * grid (n*n channels), the library's FFT workspace for it and the sorted
- * point tables on the current device.  Synchronous. */
+ * points per axis (MBO_ERR_UNSUPPORTED_SIZE above 2048).  Allocates the
+ * grid (n*n channels; MBO_F32: the box of it that holds the points'
+ * footprints), the FFT workspace for it and the sorted point tables on the
+ * current device.  Synchronous. */
 MBO_API mbo_status mbo_surface_create(mbo_surface* out, int64_t nq, const double* xq,
                                       const double* wq, const double* xc, int n, double tau,
                                       double eps, mbo_dtype dtype);
