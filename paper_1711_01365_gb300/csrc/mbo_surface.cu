@@ -11,10 +11,10 @@
 //   k_spread   type-1 spreading: source q adds w_q A(x_q^c) phi(2 (j - u_q) / W) to
 //              the W^3 grid points j around its grid coordinate u_q (phi of a
 //              vector: the product of its three coordinates' factors).
-//   (the library's 3-D FFT diffusion with the per-axis multiplier
+//   (3-D FFT diffusion with the per-axis multiplier
 //              nf (h / 2 pi) win(k) e^{-k^2 h^2 tau} / psi(k)^2, psi the kernel's
-//              Fourier transform: forward FFT, multiplier, inverse FFT, in one
-//              call of the torus path)
+//              Fourier transform: forward FFT, multiplier, inverse FFT; FP32 on
+//              the box of the points, mbo_box.cuh, FP64 one call of the torus path)
 //   k_interp   type-2 interpolation: target t sums the phi-weighted grid values
 //              around its coordinate.
 //   k_sproject projection of every target (Lemma 1.1) with the step statistics.
@@ -26,13 +26,15 @@
 //
 // Points whose footprints (the W^3 grid points spread to or read from) start
 // at the same grid point share their footprint, and the plan sorts them into
-// such groups once (the geometry is fixed).  Spreading: one warp per group of
-// sources, a lane per footprint column (x, y) holding the W points along z for
-// CG channels in registers; the group's sources are summed there and added once
-// to a shared-memory tile of the group's bin of kBin^3 cells, which goes to the
-// grid at the end.  Interpolation: one block per group of targets stages the
-// footprint values in shared memory once and evaluates every target of the
-// group from them, a thread per target.
+// such groups once (the geometry is fixed).  Spreading (k_spread): one warp per
+// group of sources, a lane per footprint column (x, y) holding the W points along
+// z for CG channels in registers; the group's sources are summed there and added
+// once to a shared-memory tile of the group's bin of kBin^3 cells, which goes to
+// the grid at the end.  FP32 at width 7 (k_spread7): the groups of a column slide
+// along z and what falls out goes straight to the grid.  Interpolation: one block
+// per group of targets stages the footprint values in shared memory once and
+// evaluates every target of the group from them (k_interp a target per thread,
+// k_interp7 two).
 #include <cuda_runtime.h>
 
 #include <algorithm>
