@@ -1213,14 +1213,9 @@ __device__ __forceinline__ bool polar3_quat_f64(const double* m, double* b, doub
   return true;
 }
 
-// n = 3: Newton, then the Jacobi construction where m is singular to working
-// precision; out of line, for the points polar3_quat_f64 leaves.
-struct MatD9 {
-  double b[9];
-  double sg;
-};
-static __device__ __noinline__ MatD9 polar3_newton_cold(const double* m) {
-  MatD9 r;
+// n = 3, FP64: Newton, then the Jacobi construction where m is singular to working
+// precision.
+__device__ __forceinline__ double polar3_newton_f64(const double* m, double* b) {
   double x[9], nx = 0.0;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -1228,8 +1223,19 @@ static __device__ __noinline__ MatD9 polar3_newton_cold(const double* m) {
     nx += x[k] * x[k];
   }
   double est = 0.0, smin;
-  r.sg = polar3_newton<16, 3>(x, r.b, est, 1e-12 * sqrt(nx), 1e-24 * nx * nx);
-  if (!(est > 1e-12 * sqrt(nx))) r.sg = polar3(x, r.b, smin);
+  double sg = polar3_newton<16, 3>(x, b, est, 1e-12 * sqrt(nx), 1e-24 * nx * nx);
+  if (!(est > 1e-12 * sqrt(nx))) sg = polar3(x, b, smin);
+  return sg;
+}
+
+// Out of line, for the points polar3_quat_f64 leaves.
+struct MatD9 {
+  double b[9];
+  double sg;
+};
+static __device__ __noinline__ MatD9 polar3_newton_cold(const double* m) {
+  MatD9 r;
+  r.sg = polar3_newton_f64(m, r.b);
   return r;
 }
 
