@@ -24,8 +24,9 @@
 //   into 31 + 31 bits, so a real product is a high product, two cross products
 //   and the upper word of the low one; a complex product sums the cross terms
 //   of both parts before the one rounding shift.
-//   Range.  Any finite input is accepted: norms outside the FP32 range take a
-//   slower pass that scales by the largest exponent first.  A sequence with a
+//   Range.  Any finite input is accepted, subnormals included: norms outside the
+//   FP32 range take a slower pass that scales by the largest exponent first, and
+//   results below 2^-1022 are rounded to subnormals as FP64 does.  A sequence with a
 //   non-finite entry gives NaN throughout, as a floating-point DFT does.
 //   W stays in FP64 between the passes.
 #pragma once
@@ -282,7 +283,7 @@ __device__ __noinline__ void fft_fx(fx2* s, L lay, int N, int M, const Plan& pl,
 // at its own rate: two conversions cost as much as two FP64 operations).
 // ---------------------------------------------------------------------------
 
-// round(d 2^k) for |d| 2^k < 2^62; k as the scale functions give it.
+// round(d 2^k) for |d| 2^k < 2^62 and d zero or normal; k as the scale functions give it.
 __device__ __forceinline__ long long fx_from(double d, int k) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(d);
   const int e = (int)(u >> 52) & 0x7ff;
@@ -295,7 +296,7 @@ __device__ __forceinline__ long long fx_from(double d, int k) {
   return (long long)u < 0 ? -v : v;
 }
 
-// v 2^e, rounded to FP64 (overflow to infinity, underflow to zero)
+// v 2^e rounded to FP64 (overflow to infinity; zero below 2^-1022)
 __device__ __forceinline__ double fx_to(long long v, int e) {
   if (v == 0) return 0.0;
   const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
@@ -307,6 +308,16 @@ __device__ __forceinline__ double fx_to(long long v, int e) {
   if (ex > 2045) b = 0x7ff0000000000000ull;
   return __longlong_as_double((long long)(b | ((unsigned long long)v & 0x8000000000000000ull)));
 }
+
+// Subnormals occur only in sequences whose scale k is large.  There the values
+// are lifted by 2^600 before fx_from and lowered again after fx_to (an FP64 multiply,
+// which rounds results below 2^-1022 as FP64 does), each in a loop of its own, so
+// that the conversions of ordinary sequences do not test for them (per element
+// that took 1 to 4% of a step).
+constexpr int kFxBad = 0x7fffffff;  // scale of a sequence with a non-finite entry
+constexpr int kFxUp = 600;
+__device__ __forceinline__ int fx_lift(int k) { return k > 960 && k != kFxBad ? kFxUp : 0; }
+__device__ __forceinline__ void fx_scale2(double2& z, double f) { z = double2{z.x * f, z.y * f}; }
 
 // A part in FP32.
 __device__ __forceinline__ float fx_float(long long v) {
@@ -320,8 +331,6 @@ __device__ __forceinline__ float fx_mod(float x, float y) {
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(big) : "f"(fabsf(x)), "f"(fabsf(y)));
   return big + 0.4142136f * fminf(fabsf(x), fabsf(y));
 }
-
-constexpr int kFxBad = 0x7fffffff;  // scale of a sequence with a non-finite entry
 
 // k such that a bound of s 2^e becomes less than 2^62, with room for the
 // roundings of the sum and of the transform (s finite, positive and normal).
@@ -337,24 +346,27 @@ __device__ __forceinline__ FxScale fx_scales(float l1, float mx, int e, int r) {
 }
 __device__ __forceinline__ bool fx_plain(float s) { return s > 1e-30f && s < 1e37f; }
 
+constexpr int kFxZero = -2000;  // below every exponent
+// floor(log2 |d|) of any d: kFxZero for zeros, 1024 for infinities and NaN
+__device__ __forceinline__ int fx_exponent(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d) & 0x7fffffffu, lo = (unsigned)__double2loint(d);
+  if (hi >= 0x00100000u) return (int)(hi >> 20) - 1023;
+  return hi ? -1011 - __clz((int)hi) : lo ? -1043 - __clz((int)lo) : kFxZero;
+}
+
 // Scales of one sequence whose FP32 norm is out of range (all threads of the
 // block call it; `each(f)` runs f over this thread's entries of the sequence).
 // red: 32 words.
 template <class Each> __device__ FxScale fx_scale_slow(Each each, int r, unsigned* red) {
-  // the largest magnitude's high word orders the exponents; 0x7ff00000: not finite
-  unsigned top = 0;
-  each([&](double2 z) {
-    top = max(top, (unsigned)__double2hiint(z.x) & 0x7fffffffu);
-    top = max(top, (unsigned)__double2hiint(z.y) & 0x7fffffffu);
-  });
-  top = __reduce_max_sync(0xffffffffu, top);
+  int e = kFxZero;
+  each([&](double2 z) { e = max(e, max(fx_exponent(z.x), fx_exponent(z.y))); });
+  e = __reduce_max_sync(0xffffffffu, e);
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (unsigned)e;
   __syncthreads();
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) top = max(top, red[w]);
-  if (top >= 0x7ff00000u) return FxScale{kFxBad, 0};
-  if (top < 0x00100000u) return FxScale{0, 0};  // zeros and denormals only
-  const int e = (int)(top >> 20) - 1023;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) e = max(e, (int)red[w]);
+  if (e == 1024) return FxScale{kFxBad, 0};
+  if (e == kFxZero) return FxScale{0, 0};
   float s = 0.f;
   each([&](double2 z) { s += fx_mod((float)scalbn(z.x, -e), (float)scalbn(z.y, -e)); });
   s = warp_sum(s);
@@ -429,14 +441,20 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
         sum += rs[0][w][q];
         top = fmaxf(top, rs[1][w][q]);
       }
-      const FxScale f = fx_plain(sum) ? fx_scales(sum, top, 0, r)
-                                      : fx_scale_slow(
-                                            [&](auto each) {
-                                              for (int x = tid; x < nx; x += T) each(sd[lay.addr(q, x)]);
-                                            },
-                                            r, slow);
+      FxScale f;
+      int up = 0;
+      if (fx_plain(sum)) {
+        f = fx_scales(sum, top, 0, r);
+      } else {
+        auto points = [&](auto each) {
+          for (int x = tid; x < nx; x += T) each(sd[lay.addr(q, x)]);
+        };
+        f = fx_scale_slow(points, r, slow);
+        up = fx_lift(f.in);
+        if (up) points([](double2& z) { fx_scale2(z, 0x1p600); });
+      }
       k[q] = f.k;
-      kin[q] = f.in;
+      kin[q] = f.in - up;
       if (tid == 0) drops[q] = f.k == kFxBad ? 0 : f.in - f.k;
     }
     for (int x = tid; x < nx; x += T) {
@@ -474,8 +492,12 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
     fft_fx(s, lay, nx, Q, t.plan[0], tw, false, drops);
     for (int x = tid; x < nx; x += T) {
 #pragma unroll
-      for (int q = 0; q < Q; ++q) W[q * P + off + x] = from_fixed(s[lay.addr(q, x)], k[q]);
+      for (int q = 0; q < Q; ++q) W[q * P + off + x] = from_fixed(s[lay.addr(q, x)], k[q] - fx_lift(k[q]));
     }
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (fx_lift(k[q]))
+        for (int x = tid; x < nx; x += T) fx_scale2(W[q * P + off + x], 0x1p-600);
     if (sp.do_stats) {
       const double tot = block_sum(defect, redd);
       double all;
@@ -501,7 +523,8 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
       for (int x = tid; x < nx; x += T) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-          const double2 z = from_fixed(s[lay.addr(q, x)], k[q]);  // swapped
+          double2 z = from_fixed(s[lay.addr(q, x)], k[q] - fx_lift(k[q]));  // swapped
+          if (fx_lift(k[q])) fx_scale2(z, 0x1p-600);
           A[(2 * q) * P + off + x] = z.y;
           if (2 * q + 1 < C) A[(2 * q + 1) * P + off + x] = z.x;
         }
@@ -515,6 +538,13 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
     const int ku = fx_unit_scale(nx);
     const int kin = t.plan[0].nst > 1 ? 61 - (32 - __clz(t.plan[0].st[0].rad - 1)) : ku;
     int bad = 0;
+    {  // the polar factor does not depend on the scale: where every plane is lifted, m stays so
+      int up = kFxUp;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) up = min(up, fx_lift(k[q]));
+#pragma unroll
+      for (int q = 0; q < Q; ++q) k[q] -= up;
+    }
     for (int x = tid; x < nx; x += T) {
       double old[C], m[C], b[C], sg;
 #pragma unroll
@@ -632,6 +662,7 @@ k_axis_fx(Geom g, Tables<double> t, double2* W, StatsPtrs sp, int axis, int ltx)
     col_fold(n, mx);
     const bool plain = fx_plain(n);
     FxScale f = plain ? fx_scales(n, mx, 0, r0) : FxScale{0, 0};
+    int up = 0;
     if (!__syncthreads_and(plain)) {
       for (int c = 0; c < tx; ++c) {
         const FxScale fc = fx_scale_slow(
@@ -642,9 +673,13 @@ k_axis_fx(Geom g, Tables<double> t, double2* W, StatsPtrs sp, int axis, int ltx)
             r0, slow);
         if (mcol == c) f = fc;
       }
+      up = fx_lift(f.in);
+      if (up)
+        for (int p = p0; p < L; p += dp) fx_scale2(sd[lay.addr(mcol, p)], 0x1p600);
     }
     k = f.k;
     if (tid < tx) drops[tid] = k == kFxBad ? 0 : f.in - k;  // thread tid owns column tid
+    f.in -= up;
     for (int p = p0; p < L; p += dp) {
       const int a = lay.addr(mcol, p);
       const double2 z = sd[a];
@@ -717,13 +752,13 @@ k_axis_fx(Geom g, Tables<double> t, double2* W, StatsPtrs sp, int axis, int ltx)
         }
       }
       if (tid < tx) drops[tid] = f.in - f.k;
-      const int sft = f.in;
+      const int sft = f.in + ge;
       for (int p = p0; p < L; p += dp) {
         const int a = lay.addr(mcol, p);
         const fx2 v = s[a];
-        // v f 2^sft: the 53-bit mantissa of f as Q60 in [1/2, 1), its exponent
+        // v f 2^sft, f in units of 2^ge: its 53-bit mantissa as Q60 in [1/2, 1), its exponent
         // joins the shift, so that small products keep their digits
-        const unsigned long long u = (unsigned long long)__double_as_longlong(gcol * gL[p]);
+        const unsigned long long u = (unsigned long long)__double_as_longlong(gm * gL[p]);
         const int fe = (int)(u >> 52) & 0x7ff;
         long long mt = (long long)(((u & 0xfffffffffffffull) | 0x10000000000000ull) << 7);
         if ((long long)u < 0) mt = -mt;
@@ -739,10 +774,15 @@ k_axis_fx(Geom g, Tables<double> t, double2* W, StatsPtrs sp, int axis, int ltx)
   if (MODE == AXIS_FGI) fft_fx(s, lay, L, tx, t.plan[axis], tw, true, drops);
   if (MODE != AXIS_ENERGY && live) {
     double2* dst = base + mcol + (long long)p0 * es;
+    const int up = fx_lift(k), e = up - k;
     for (int p = p0; p < L; p += dp, dst += gstep) {
       const fx2 v = s[lay.addr(mcol, p)];
-      const double re = fx_to(MODE == AXIS_FWD ? v.x : v.y, -k), im = fx_to(MODE == AXIS_FWD ? v.y : v.x, -k);
+      const double re = fx_to(MODE == AXIS_FWD ? v.x : v.y, e), im = fx_to(MODE == AXIS_FWD ? v.y : v.x, e);
       *dst = k == kFxBad ? double2{nan, nan} : double2{re, im};
+    }
+    if (up) {
+      dst = base + mcol + (long long)p0 * es;
+      for (int p = p0; p < L; p += dp, dst += gstep) fx_scale2(*dst, 0x1p-600);
     }
   }
   if ((MODE == AXIS_FGI || MODE == AXIS_ENERGY) && sp.do_stats) {
