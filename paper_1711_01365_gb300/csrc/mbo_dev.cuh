@@ -1076,141 +1076,108 @@ static __device__ __noinline__ double polar4_jacobi(const double* m, double* b, 
   return want;
 }
 
-// n = 3, FP64: the polar factor from an FP32 quaternion refined in FP64.  FP64
-// instructions issue at 1/64 of the FP32 rate on this GPU, and the scaled Newton
-// iteration needs about 500 of them per point; here all but some 110 are FP32.
-//
-// For a = sg m, sg the sign of det m, the nearest rotation R(q) maximises
-// q^t K q over unit quaternions (Horn 1987; K as in polar3_quat), so q is the
-// eigenvector of the largest eigenvalue of the symmetric 4x4 matrix K.  With q
-// from polar3_quat_vec in FP32 (error about eps32 / gap), a correction step is
-//   r = K q - mu q (FP64, mu the Rayleigh quotient),  (K - mu) d = -r, d orthogonal to q,
-// whose matrix and solution only need a few digits: mu I - K + c q q^t is positive
-// definite for c > 0 (its smallest eigenvalue is the gap l1 - l2 = 2 (s2 + s3)),
-// factored once in FP32 and used by every step.  A step takes the error e to
-// about eps32 cond e, cond = |K| / gap: two steps reach FP64 rounding.  They stop
-// once d is at most kQuatSettled, when what is left is below rounding.
-//
-// Taken where the class and the eigenvector are clear in FP32: |det m| above
-// kQuatDet |m|^3 and the gap bound of the quaternion form at least kQuatGap64;
-// elsewhere (and out of the FP32 range) it returns false and the caller goes on
-// with Newton.  Against polar factors in extended precision its error is 1.4 times
-// the iteration's (rms 1.5e-16 and 1.1e-16 over 256x256 random matrices), below the
-// diffusion's: a whole 1024x1024 step is off by 6.0e-16 (7.5e-16 with Newton and
-// floating-point transforms).  k_project, which only projects, keeps the iteration.
-constexpr float kQuatDet = 1e-4f;
-constexpr float kQuatGap64 = 0.02f;
-constexpr double kQuatSettled = 2e-11;
+// n = 3, FP64: the scaled Newton iteration of polar_newton, its coefficients from
+// an FP32 copy.  FP64 instructions issue at 1/64 of the FP32 rate on this GPU
+// (an instruction more per point: 1.85 us at 1024^2), and polar_newton needs about
+// 450 of them: the norms that set zeta, their 18 conversions per step and the
+// determinants of the scaled phase go into coefficients that need FP32 only.
+// Here the same steps run on an FP32 copy x, which supplies r of
+//   X <- X + r cof X,  r = 1 / (zeta^2 det)
+// (X is left scaled: a step leaves singular values (2 / zeta) (zeta s + 1 /
+// (zeta s)) / 2, the parenthesis at least 1, so x also tells how far the step
+// came); 28 FP64 instructions a step, one step where m is close to a multiple of
+// an orthogonal matrix and two to four on random matrices.  X is brought to
+// scale 1 and finished by unscaled steps in FP64, usually two of 36 and 32
+// instructions.
+//   Error.  The polar factor of X stays that of m whatever r is, up to the
+// rounding of the steps; m itself enters unrounded, so an ill-conditioned m
+// loses only what cof m loses.  Over random and over graded matrices (s =
+// (1, 0.05, <= 0.05)), against extended precision, |error|_F: RMS 1.48e-16 and 2.0e-16
+// (polar_newton 1.69e-16 and 2.2e-16); mean defect of orthogonality 1.34e-16
+// (1.45e-16).
+//   Last step.  After an unscaled step every singular value is 1 + d, d >= 0, so
+// |det X| - 1 bounds the d: at kNewtonLast the next step ends at d^2 / 2 below
+// 2e-17, and 2 - |det| is 1 / |det| to the same.
+// Taken where FP32 holds m and its class is clear: |det m| above
+// kNewtonDet |m|^3 (the smallest singular value is then above 1e-4 |m|, which FP32
+// resolves); elsewhere false, and the caller goes on with polar_newton.
+constexpr float kNewtonDet = 1e-4f;
+constexpr float kNewtonNear = 1.5e-4f;  // sum of s^2 - 1 that ends the scaled steps
+constexpr double kNewtonLast = 6e-9;
 
-__device__ __forceinline__ bool polar3_quat_f64(const double* m, double* b, double& sg) {
-  float f[9], n2 = 0.f;
+// x / 2 in the integer pipe (subnormals, below any rounding here, stay)
+__device__ __forceinline__ double half_bits(double x) {
+  const int hi = __double2hiint(x);
+  return __hiloint2double((hi & 0x7ff00000) ? hi - 0x00100000 : hi, __double2loint(x));
+}
+
+__device__ __forceinline__ bool polar3_guided(const double* m, double* b, double& sg) {
+  float x[9], c[9], nx = 0.f;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    f[k] = (float)m[k];
-    n2 += f[k] * f[k];
+    x[k] = (float)m[k];
+    nx += x[k] * x[k];
   }
-  if (!(n2 > 1e-24f && n2 < 1e24f)) return false;  // out of range, or not finite
-  const float inv = rsqrtf(n2);
+  if (!(nx > 1e-24f && nx < 1e24f)) return false;  // out of range, or not finite
+  const float inv = rsqrtf(nx);
+  nx = 0.f;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) f[k] *= inv;
-  const float det = f[0] * (f[4] * f[8] - f[5] * f[7]) - f[1] * (f[3] * f[8] - f[5] * f[6]) +
-                    f[2] * (f[3] * f[7] - f[4] * f[6]);
-  if (!(fabsf(det) > kQuatDet)) return false;
-  const float sf = det >= 0.f ? 1.f : -1.f;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) f[k] *= sf;
-  float v[4], l1;
-  if (!(quat_vec(f, v, l1) >= kQuatGap64)) return false;
-  sg = (double)sf;
-  {
-    const float in = rsqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] *= in;
+  for (int k = 0; k < 9; ++k) {
+    x[k] *= inv;
+    nx += x[k] * x[k];
   }
-  // FP32 factor L D L^t of mu I - K + q q^t (K scaled to |a|_F = 1)
-  float l10, l20, l30, l21, l31, l32, d0, d1, d2, d3;
-  {
-    const float k00 = f[0] + f[4] + f[8], k11 = f[0] - f[4] - f[8], k22 = -f[0] + f[4] - f[8],
-                k33 = -f[0] - f[4] + f[8];
-    const float a00 = l1 - k00 + v[0] * v[0], a11 = l1 - k11 + v[1] * v[1], a22 = l1 - k22 + v[2] * v[2],
-                a33 = l1 - k33 + v[3] * v[3];
-    const float a10 = v[0] * v[1] - (f[7] - f[5]), a20 = v[0] * v[2] - (f[2] - f[6]),
-                a30 = v[0] * v[3] - (f[3] - f[1]), a21 = v[1] * v[2] - (f[1] + f[3]),
-                a31 = v[1] * v[3] - (f[2] + f[6]), a32 = v[2] * v[3] - (f[5] + f[7]);
-    d0 = __frcp_rn(a00);
-    l10 = a10 * d0, l20 = a20 * d0, l30 = a30 * d0;
-    const float b11 = a11 - l10 * a10, b21 = a21 - l20 * a10, b31 = a31 - l30 * a10;
-    const float b22 = a22 - l20 * a20, b32 = a32 - l30 * a20, b33 = a33 - l30 * a30;
-    d1 = __frcp_rn(b11);
-    l21 = b21 * d1, l31 = b31 * d1;
-    const float c22 = b22 - l21 * b21, c32 = b32 - l31 * b21, c33 = b33 - l31 * b31;
-    d2 = __frcp_rn(c22);
-    l32 = c32 * d2;
-    d3 = __frcp_rn(c33 - l32 * c32);
-  }
-  // K of sg m; the signs are flipped in the integer pipe
-  auto sgn = [neg = sf < 0.f](double x) {
-    return neg ? __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x)) : x;
-  };
-  const double t0 = sgn(m[0]), t4 = sgn(m[4]), t8 = sgn(m[8]);
-  const double p48 = t4 + t8, m48 = t4 - t8;
-  const double K00 = t0 + p48, K11 = t0 - p48, K22 = m48 - t0, K33 = -(t0 + m48);
-  const double K01 = sgn(m[7] - m[5]), K02 = sgn(m[2] - m[6]), K03 = sgn(m[3] - m[1]);
-  const double K12 = sgn(m[1] + m[3]), K13 = sgn(m[2] + m[6]), K23 = sgn(m[5] + m[7]);
-  double q[4] = {(double)v[0], (double)v[1], (double)v[2], (double)v[3]};
-  bool settled = false;
+  float det = cofactor3(x, c);
+  if (!(fabsf(det) > kNewtonDet)) return false;
+  const bool neg = det < 0.f;
+  sg = neg ? -1.0 : 1.0;
+  double X[9], C[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) X[k] = m[k];
+  float scale = 1.f;  // of x
 #pragma unroll 1
-  for (int it = 0; it < 4; ++it) {
-    const double y0 = K00 * q[0] + K01 * q[1] + K02 * q[2] + K03 * q[3];
-    const double y1 = K01 * q[0] + K11 * q[1] + K12 * q[2] + K13 * q[3];
-    const double y2 = K02 * q[0] + K12 * q[1] + K22 * q[2] + K23 * q[3];
-    const double y3 = K03 * q[0] + K13 * q[1] + K23 * q[2] + K33 * q[3];
-    // mu only has to make r orthogonal to q up to the size of d: q q within
-    // 1e-6 of 1 would leave mu 1e-6 off, so divide by it (to first order: the
-    // norm is 1 + e with e below 1e-6, and e^2 is below rounding)
-    const double qq = q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
-    const double mu = (y0 * q[0] + y1 * q[1] + y2 * q[2] + y3 * q[3]) * (2.0 - qq);
-    const float r0 = (float)(y0 - mu * q[0]) * inv, r1 = (float)(y1 - mu * q[1]) * inv;
-    const float r2 = (float)(y2 - mu * q[2]) * inv, r3 = (float)(y3 - mu * q[3]) * inv;
-    const float z1 = r1 - l10 * r0;
-    const float z2 = r2 - l20 * r0 - l21 * z1;
-    const float z3 = r3 - l30 * r0 - l31 * z1 - l32 * z2;
-    const float x3 = z3 * d3;
-    const float x2 = z2 * d2 - l32 * x3;
-    const float x1 = z1 * d1 - l21 * x2 - l31 * x3;
-    const float x0 = r0 * d0 - l10 * x1 - l20 * x2 - l30 * x3;
-    q[0] += (double)x0;
-    q[1] += (double)x1;
-    q[2] += (double)x2;
-    q[3] += (double)x3;
-    const float dmax = fmaxf(fmaxf(fabsf(x0), fabsf(x1)), fmaxf(fabsf(x2), fabsf(x3)));
-    if (dmax <= (float)kQuatSettled) {
-      settled = true;
-      break;
+  for (int it = 0; it < 8; ++it) {
+    float nc = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) nc += c[k] * c[k];
+    const float iz2 = sqrtf(__fdividef(det * det * nx, nc));  // 1 / zeta^2
+    const float r = __fdividef(iz2, det);
+    (void)cofactor3(X, C);
+    const double rd = (double)(r * inv);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) X[k] = fma(rd, C[k], X[k]);
+    nx = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      x[k] = fmaf(r, c[k], x[k]);
+      nx += x[k] * x[k];
     }
+    scale = 2.f * sqrtf(iz2);
+    if (nx <= (3.f + kNewtonNear) * (scale * scale)) break;
+    det = cofactor3(x, c);
   }
-  if (!settled) return false;
-  // R(q) / |q|^2.  |q|^2 = 1 + e with |e| of the FP32 rounding, so 1 / |q|^2 is 1 + c,
-  // c = e^2 - e, to rounding; added as x + x c, which rounds once where x (1 + c)
-  // rounds twice (orthogonality defect over random q: 1.0e-15 at most -> 6.9e-16)
-  const double ww = q[0] * q[0], yy = q[2] * q[2];
-  const double wx = fma(q[1], q[1], ww), yz = fma(q[3], q[3], yy);
-  const double wmx = fma(-q[1], q[1], ww), ymz = fma(-q[3], q[3], yy);
-  const double e = (wx - 1.0) + yz, c = fma(e, e, -e), c2 = c + c;
-  const double t00 = sgn(wx - yz), t11 = sgn(wmx + ymz), t22 = sgn(wmx - ymz);
-  b[0] = fma(t00, c, t00);
-  b[4] = fma(t11, c, t11);
-  b[8] = fma(t22, c, t22);
-  const double hx = sgn(fma(q[1], c2, q[1] + q[1])), hy = sgn(fma(q[2], c2, q[2] + q[2])),
-               hz = sgn(fma(q[3], c2, q[3] + q[3]));
-  const double xy = hx * q[2], xz = hx * q[3], yz2 = hy * q[3];
-  b[1] = xy - hz * q[0];
-  b[3] = xy + hz * q[0];
-  b[2] = xz + hy * q[0];
-  b[6] = xz - hy * q[0];
-  b[5] = yz2 - hx * q[0];
-  b[7] = yz2 + hx * q[0];
-  return true;
+  const double up = (double)__fdividef(inv, scale);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) X[k] *= up;
+  bool last = false;
+#pragma unroll 1
+  for (int it = 0; it < 6 && !last; ++it) {
+    const double ad = fabs(cofactor3(X, C));
+    last = it > 0 && ad - 1.0 <= kNewtonLast;
+    double r;
+    if (last) {
+      r = 2.0 - ad;
+    } else {
+      r = (double)__frcp_rn((float)ad);
+      r = r * (2.0 - ad * r);
+    }
+    r = half_bits(r);
+    if (neg) r = -r;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) X[k] = fma(r, C[k], half_bits(X[k]));
+  }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) b[k] = X[k];
+  return last;
 }
 
 // n = 3, FP64: Newton, then the Jacobi construction where m is singular to working
@@ -1228,20 +1195,34 @@ __device__ __forceinline__ double polar3_newton_f64(const double* m, double* b) 
   return sg;
 }
 
-// Out of line, for the points polar3_quat_f64 leaves.
+// Out of line, for the points polar3_guided leaves.  A matrix beyond the FP32 range is
+// scaled first, by a power of two: the polar factor does not depend on it.
 struct MatD9 {
   double b[9];
   double sg;
 };
 static __device__ __noinline__ MatD9 polar3_newton_cold(const double* m) {
   MatD9 r;
-  r.sg = polar3_newton_f64(m, r.b);
+  double big = 0.0, x[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    x[k] = m[k];
+    big = fmax(big, fabs(m[k]));
+  }
+  if ((big < 1e-12 || big > 2e11) && big > 0.0 && isfinite(big)) {
+    const int e = ilogb(big);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) x[k] = scalbn(m[k], -e);
+    if (polar3_guided(x, r.b, r.sg)) return r;
+  }
+  r.sg = polar3_newton_f64(x, r.b);
   return r;
 }
 
-// FP64 projection used by the FP64 path and by the FP32 path's
-// re-projection: for n = 3 the refined quaternion form, else and elsewhere Newton, and the one-sided Jacobi construction for matrices
-// that are singular to working precision (rank-deficient ties included).
+// FP64 projection used by the FP64 path and by the FP32 path's re-projection:
+// Newton (n = 3: guided by FP32 where that is possible), and the one-sided
+// Jacobi construction for matrices that are singular to working precision
+// (rank-deficient ties included).
 template <int NM> __device__ __forceinline__ double polar_f64(const double* m, double* b) {
   if constexpr (NM == 4) {
     double nx = 0.0;
@@ -1260,7 +1241,7 @@ template <int NM> __device__ __forceinline__ double polar_f64(const double* m, d
     return polar4_jacobi(m, b, smin);
   } else if constexpr (NM == 3) {
     double sg;
-    if (polar3_quat_f64(m, b, sg)) return sg;
+    if (polar3_guided(m, b, sg)) return sg;
     const MatD9 r = polar3_newton_cold(m);
 #pragma unroll
     for (int k = 0; k < 9; ++k) b[k] = r.b[k];

@@ -608,12 +608,7 @@ k_project(long long P, const R* At, R* B, int8_t* ds, R fb_sigma) {
     R m[C], b[C], sg;
 #pragma unroll
     for (int c = 0; c < C; ++c) m[c] = At[c * P + x];
-    if constexpr (NM == 3 && sizeof(R) == 8) {
-      // the iteration: no diffusion error beside which the quaternion form's last bits vanish
-      sg = polar3_newton_f64(m, b);
-    } else {
-      if (!project_point<NM>(m, b, sg, fb_sigma)) sg = project_point_f64<NM>(m, b);
-    }
+    if (!project_point<NM>(m, b, sg, fb_sigma)) sg = project_point_f64<NM>(m, b);
 #pragma unroll
     for (int c = 0; c < C; ++c) B[c * P + x] = b[c];
     if (ds) ds[x] = (sg > R(0)) ? 1 : -1;
