@@ -332,6 +332,19 @@ __device__ __forceinline__ float fx_mod(float x, float y) {
   return big + 0.4142136f * fminf(fabsf(x), fabsf(y));
 }
 
+__device__ __forceinline__ bool fx_nonzero(double d) {
+  return (((unsigned)__double2hiint(d) << 1) | (unsigned)__double2loint(d)) != 0;
+}
+// The bound of an entry that norms are summed from: positive for every entry but
+// zero, so that a norm is 0 for a sequence of zeros only.  Those are common (dead
+// columns of a ragged tile, constant channels, grid outside a surface's points)
+// and need no scale.
+constexpr float kFxTiny = 1.4e-45f;
+__device__ __forceinline__ float fx_norm(double2 z) {
+  const float a = fx_mod((float)z.x, (float)z.y);
+  return a == 0.f && (fx_nonzero(z.x) || fx_nonzero(z.y)) ? kFxTiny : a;
+}
+
 // k such that a bound of s 2^e becomes less than 2^62, with room for the
 // roundings of the sum and of the transform (s finite, positive and normal).
 __device__ __forceinline__ int fx_scale(float s, int e) { return 61 - ilogbf(s * 1.002f) - e; }
@@ -341,10 +354,12 @@ struct FxScale {
   int k, in;
 };
 __device__ __forceinline__ FxScale fx_scales(float l1, float mx, int e, int r) {
+  if (l1 == 0.f) return FxScale{0, 0};
   const int k = fx_scale(l1, e);
   return FxScale{k, max(k, fx_scale(mx * (float)r, e))};
 }
-__device__ __forceinline__ bool fx_plain(float s) { return s > 1e-30f && s < 1e37f; }
+// Whether the FP32 norm gives the scale.
+__device__ __forceinline__ bool fx_plain(float s) { return s == 0.f || (s > 1e-30f && s < 1e37f); }
 
 constexpr int kFxZero = -2000;  // below every exponent
 // floor(log2 |d|) of any d: kFxZero for zeros, 1024 for infinities and NaN
@@ -418,7 +433,7 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         const double2 z = sd[lay.addr(q, x)];
-        const float a = fx_mod((float)z.x, (float)z.y);
+        const float a = fx_norm(z);
         n[q] += a;
         mx[q] = fmaxf(mx[q], a);
       }
@@ -655,7 +670,7 @@ k_axis_fx(Geom g, Tables<double> t, double2* W, StatsPtrs sp, int axis, int ltx)
     float n = 0.f, mx = 0.f;
     for (int p = p0; p < L; p += dp) {
       const double2 z = sd[lay.addr(mcol, p)];
-      const float a = fx_mod((float)z.x, (float)z.y);
+      const float a = fx_norm(z);
       n += a;
       mx = fmaxf(mx, a);
     }
@@ -665,6 +680,9 @@ k_axis_fx(Geom g, Tables<double> t, double2* W, StatsPtrs sp, int axis, int ltx)
     int up = 0;
     if (!__syncthreads_and(plain)) {
       for (int c = 0; c < tx; ++c) {
+        float nc = 0.f;  // column c's norm, as col_fold left its parts
+        for (int w = 0; w < (T >> 5); ++w) nc += rs[0][w][c];
+        if (fx_plain(nc)) continue;
         const FxScale fc = fx_scale_slow(
             [&](auto each) {
               if (mcol == c)
@@ -728,14 +746,16 @@ k_axis_fx(Geom g, Tables<double> t, double2* W, StatsPtrs sp, int axis, int ltx)
       float n = 0.f, mx = 0.f;
       for (int p = p0; p < L; p += dp) {
         const fx2 v = s[lay.addr(mcol, p)];
-        const float a = fx_mod(fx_float(v.x), fx_float(v.y)) * fabsf((float)(gm * gL[p]));
+        const double gp = gm * gL[p];
+        float a = fx_mod(fx_float(v.x), fx_float(v.y)) * fabsf((float)gp);
+        if (a == 0.f && (v.x | v.y) != 0 && fx_nonzero(gp)) a = kFxTiny;
         n += a;
         mx = fmaxf(mx, a);
       }
       col_fold(n, mx);
       FxScale f = n > 1e-20f ? fx_scales(n, mx, ge, r_inv) : FxScale{0, 0};
-      if (!__syncthreads_and(n > 1e-20f || k == kFxBad)) {
-        // zeros, or products below the FP32 range: the norm in FP64
+      if (!__syncthreads_and(n > 1e-20f || n == 0.f || k == kFxBad)) {
+        // products below the FP32 range: the norm in FP64
         double nd = 0.0;
         for (int p = p0; p < L; p += dp) {
           const fx2 v = s[lay.addr(mcol, p)];
