@@ -1087,8 +1087,7 @@ static __device__ __noinline__ double polar4_jacobi(const double* m, double* b, 
 // (zeta s)) / 2, the parenthesis at least 1, so x also tells how far the step
 // came); 28 FP64 instructions a step, one step where m is close to a multiple of
 // an orthogonal matrix and two to four on random matrices.  X is brought to
-// scale 1 and finished by unscaled steps in FP64, usually two of 36 and 32
-// instructions.
+// scale 1 and finished by unscaled steps in FP64, usually two of 33 instructions.
 //   Error.  The polar factor of X stays that of m whatever r is, up to the
 // rounding of the steps; m itself enters unrounded, so an ill-conditioned m
 // loses only what cof m loses.  Over random and over graded matrices (s =
@@ -1096,8 +1095,8 @@ static __device__ __noinline__ double polar4_jacobi(const double* m, double* b, 
 // (polar_newton 1.69e-16 and 2.2e-16); mean defect of orthogonality 1.34e-16
 // (1.45e-16).
 //   Last step.  After an unscaled step every singular value is 1 + d, d >= 0, so
-// |det X| - 1 bounds the d: at kNewtonLast the next step ends at d^2 / 2 below
-// 2e-17, and 2 - |det| is 1 / |det| to the same.
+// e = |det X| - 1 bounds the d: at kNewtonLast the next step ends at d^2 / 2 below
+// 2e-17.  1 / |det X| is 1 - e + e^2 to e^3.
 // Taken where FP32 holds m and its class is clear: |det m| above
 // kNewtonDet |m|^3 (the smallest singular value is then above 1e-4 |m|, which FP32
 // resolves); elsewhere false, and the caller goes on with polar_newton.
@@ -1161,16 +1160,9 @@ __device__ __forceinline__ bool polar3_guided(const double* m, double* b, double
   bool last = false;
 #pragma unroll 1
   for (int it = 0; it < 6 && !last; ++it) {
-    const double ad = fabs(cofactor3(X, C));
-    last = it > 0 && ad - 1.0 <= kNewtonLast;
-    double r;
-    if (last) {
-      r = 2.0 - ad;
-    } else {
-      r = (double)__frcp_rn((float)ad);
-      r = r * (2.0 - ad * r);
-    }
-    r = half_bits(r);
+    const double ad = fabs(cofactor3(X, C)), e = ad - 1.0;
+    last = it > 0 && __double_as_longlong(ad) <= __double_as_longlong(1.0 + kNewtonLast);
+    double r = half_bits(fma(e, e - 1.0, 1.0));  // 1 / (1 + e) to e^3
     if (neg) r = -r;
 #pragma unroll
     for (int k = 0; k < 9; ++k) X[k] = fma(r, C[k], half_bits(X[k]));
@@ -1195,14 +1187,20 @@ __device__ __forceinline__ double polar3_newton_f64(const double* m, double* b) 
   return sg;
 }
 
-// Out of line, for the points polar3_guided leaves.  A matrix beyond the FP32 range is
-// scaled first, by a power of two: the polar factor does not depend on it.
+// Out of line: the points polar3_guided leaves, and the FP32 path's re-projection
+// (inlined there, either iteration took the kernels from 80 registers to 96 and more).
 struct MatD9 {
   double b[9];
   double sg;
 };
 static __device__ __noinline__ MatD9 polar3_newton_cold(const double* m) {
   MatD9 r;
+  r.sg = polar3_newton_f64(m, r.b);
+  return r;
+}
+// A matrix beyond the FP32 range is scaled first, by a power of two: the polar factor
+// does not depend on it.
+static __device__ __noinline__ MatD9 polar3_cold(const double* m) {
   double big = 0.0, x[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -1213,10 +1211,10 @@ static __device__ __noinline__ MatD9 polar3_newton_cold(const double* m) {
     const int e = ilogb(big);
 #pragma unroll
     for (int k = 0; k < 9; ++k) x[k] = scalbn(m[k], -e);
+    MatD9 r;
     if (polar3_guided(x, r.b, r.sg)) return r;
   }
-  r.sg = polar3_newton_f64(x, r.b);
-  return r;
+  return polar3_newton_cold(x);
 }
 
 // FP64 projection used by the FP64 path and by the FP32 path's re-projection:
@@ -1242,7 +1240,7 @@ template <int NM> __device__ __forceinline__ double polar_f64(const double* m, d
   } else if constexpr (NM == 3) {
     double sg;
     if (polar3_guided(m, b, sg)) return sg;
-    const MatD9 r = polar3_newton_cold(m);
+    const MatD9 r = polar3_cold(m);
 #pragma unroll
     for (int k = 0; k < 9; ++k) b[k] = r.b[k];
     return r.sg;

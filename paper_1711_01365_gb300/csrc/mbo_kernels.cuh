@@ -66,13 +66,21 @@ template <int NM> __device__ __noinline__ ProjV<NM> quat_cold(MatV<NM> m, float 
 
 template <int NM> __device__ __noinline__ ProjV<NM> f64_cold(MatV<NM> m) {
   constexpr int C = NM * NM;
-  double md[C], bd[C];
+  double md[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) md[c] = (double)m.v[c];
   ProjV<NM> r;
-  r.sg = (float)polar_f64<NM>(md, bd);
+  if constexpr (NM == 3) {
+    const MatD9 d = polar3_newton_cold(md);
+    r.sg = (float)d.sg;
 #pragma unroll
-  for (int c = 0; c < C; ++c) r.b[c] = (float)bd[c];
+    for (int c = 0; c < C; ++c) r.b[c] = (float)d.b[c];
+  } else {
+    double bd[C];
+    r.sg = (float)polar_f64<NM>(md, bd);
+#pragma unroll
+    for (int c = 0; c < C; ++c) r.b[c] = (float)bd[c];
+  }
   r.gap = 0.f;
   return r;
 }
