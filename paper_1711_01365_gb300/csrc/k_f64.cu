@@ -10,9 +10,9 @@ template <int NM, int MODE>
 cudaError_t row_fx(const Geom& g, const Tables<double>& t, const double* Ain, double* A, void* W,
                    const StatsPtrs& sp, int threads, cudaStream_t s, bool prepare_only = false) {
   auto k = k_row_fx<NM, MODE>;
-  static size_t done = 0;
+  static SmemLimit limit;
   const size_t smem = row_smem_bytes(g, sizeof(double), false);
-  const cudaError_t e = set_smem(k, smem, done);
+  const cudaError_t e = raise_smem(k, smem, limit);
   if (e != cudaSuccess || prepare_only) return e;
   int rows = g.nz * g.ny;
   if (MODE == ROW_INV_PROJECT_FWD) {
@@ -48,9 +48,9 @@ template <int MODE>
 cudaError_t axis_fx(const Geom& g, const Tables<double>& t, void* W, const StatsPtrs& sp, int axis, int tx,
                     int threads, cudaStream_t s, bool prepare_only = false) {
   auto k = k_axis_fx<MODE>;
-  static size_t done = 0;
+  static SmemLimit limit;
   const size_t smem = axis_smem_bytes(axis == 1 ? g.ny : g.nz, tx, sizeof(double));
-  const cudaError_t e = set_smem(k, smem, done);
+  const cudaError_t e = raise_smem(k, smem, limit);
   if (e != cudaSuccess || prepare_only) return e;
   int ltx = 0;
   while ((1 << ltx) < tx) ++ltx;

@@ -11,20 +11,18 @@ cudaError_t wrow_nm(const Geom& g, const Tables<float>& t, const float* Ain, flo
   constexpr bool CAN_PERS = MODE == ROW_INV_PROJECT_FWD;
   auto k = k_wrow<NM, MODE, N, false, 1>;
   auto kp = k_wrow<NM, MODE, N, CAN_PERS, 1>;
-  static size_t done = 0, done_p = 0;
-  static int resident = 0;  // blocks of this kernel that fit on the device at once
-  static int sms = 0;
+  static SmemLimit limit, limit_p;
+  static DeviceCount fits;
   const size_t smem = wrow_smem_bytes(g, N, MODE == ROW_INV_PROJECT_FWD);
-  cudaError_t e = set_smem_once(k, smem, done);
-  if (e == cudaSuccess && CAN_PERS) e = set_smem_once(kp, smem, done_p);
+  cudaError_t e = raise_smem(k, smem, limit);
+  if (e == cudaSuccess && CAN_PERS) e = raise_smem(kp, smem, limit_p);
   if (e != cudaSuccess) return e;
-  if (!resident) {
-    int dev = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int dev = current_device(), sms = device_sms(dev);
+  const int resident = fits.get(dev, [&] {  // blocks of this kernel that fit on the device at once
+    int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, wrow_threads(N, NM), smem);
-    resident = sms * (per_sm > 0 ? per_sm : 1);
-  }
+    return sms * (per_sm > 0 ? per_sm : 1);
+  });
   constexpr bool CAN_HELP = MODE == ROW_INV_PROJECT_FWD && wrow_helpers(N, NM) > 1;
   if constexpr (CAN_HELP) {
     if (prepare_only && (e = launch_wrow_small(g, t, A, W, sp, fb, 0, smem, s, true)) != cudaSuccess) return e;
@@ -84,9 +82,8 @@ size_t wrow_smem_bytes(const Geom& g, int N, bool fallback) {
 namespace {
 template <int NM, int N> double wrow_waves_nm(const Geom& g) {
   auto k = k_wrow<NM, ROW_INV_PROJECT_FWD, N, false, 1>;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms(current_device());
+  int per_sm = 0;
   const size_t smem = wrow_smem_bytes(g, N, true);
   // a shape that does not fit is rejected by the caller; leave no error behind
   if ((smem > 48 * 1024 &&

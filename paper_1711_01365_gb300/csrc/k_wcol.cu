@@ -279,27 +279,24 @@ k_wcol(Geom g, Tables<float> t, const __grid_constant__ CUtensorMap tm, StatsPtr
   }
 }
 
-// Blocks of a kernel that fit on one SM, and the SM count (cached per kernel).
-template <typename K> int persistent_blocks(K kernel, int threads, size_t smem, int& per_sm) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  per_sm = 0;
+// Blocks of a kernel that fit on the device at once.
+template <typename K> int persistent_blocks(K kernel, int threads, size_t smem, int dev) {
+  int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-  if (per_sm < 1) per_sm = 1;
-  return sms * per_sm;
+  return device_sms(dev) * (per_sm > 0 ? per_sm : 1);
 }
 
 template <int MODE, int L, int TX, int NBUF>
 cudaError_t wcol_m(const Geom& g, const Tables<float>& t, const CUtensorMap* tm, const StatsPtrs& sp,
                    int axis, cudaStream_t s, bool prepare_only, const void* pf, long long pf_bytes) {
   auto k = k_wcol<MODE, L, TX, NBUF>;
-  static size_t done = 0;
-  static int slots = 0, per_sm = 0;
+  static SmemLimit limit;
+  static DeviceCount fits;
   const size_t smem = wcol_smem<L, TX>(NBUF);
-  cudaError_t e = set_smem_once(k, smem, done);
+  cudaError_t e = raise_smem(k, smem, limit);
   if (e != cudaSuccess) return e;
-  if (!slots) slots = persistent_blocks(k, WcolShape<L, TX>::NT, smem, per_sm);
+  const int dev = current_device();
+  const int slots = fits.get(dev, [&] { return persistent_blocks(k, WcolShape<L, TX>::NT, smem, dev); });
   if (prepare_only) return cudaSuccess;
   if (!tm) return cudaErrorInvalidValue;
   const int nouter = axis == 1 ? g.nz : g.ny;

@@ -11,8 +11,8 @@ cudaError_t small_nm(const Geom& g, const Tables<float>& t, float* A, void* W, c
   constexpr int HX = wrow_helpers(N, NM);
   if constexpr (HX > 1) {
     auto k = k_wrow<NM, ROW_INV_PROJECT_FWD, N, false, HX>;
-    static size_t done = 0;
-    const cudaError_t e = set_smem_once(k, smem, done);
+    static SmemLimit limit;
+    const cudaError_t e = raise_smem(k, smem, limit);
     if (e != cudaSuccess || prepare_only) return e;
     return launch_pdl(k, blocks, wrow_threads(N, NM) * HX, smem, s, g, t, (const float*)nullptr, A,
                       static_cast<float2*>(W), sp, fb, 0);

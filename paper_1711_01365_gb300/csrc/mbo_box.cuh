@@ -193,18 +193,21 @@ template <int MODE> __global__ void __launch_bounds__(kBoxThreads) k_box_axis(Bo
   }
 }
 
+inline cudaError_t box_axis_smem(size_t bytes) {
+  static SmemLimit axis[3];
+  cudaError_t e = raise_smem(k_box_axis<AXIS_FWD>, bytes, axis[0]);
+  if (e == cudaSuccess) e = raise_smem(k_box_axis<AXIS_FGI>, bytes, axis[1]);
+  if (e == cudaSuccess) e = raise_smem(k_box_axis<AXIS_INV>, bytes, axis[2]);
+  return e;
+}
+
 template <int NM> cudaError_t box_run(const BoxDiffusion& b, float* F, cudaStream_t st) {
   const size_t rs = (size_t)b.Q * row_pad(b.nf) * sizeof(float2);
   const size_t as = (size_t)row_pad(b.nf) * kBoxTx * sizeof(float2);
-  auto grow = [](auto k, size_t bytes) {
-    return bytes > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
-                             : cudaSuccess;
-  };
-  cudaError_t e = grow(k_box_row<NM, false>, rs);
-  if (e == cudaSuccess) e = grow(k_box_row<NM, true>, rs);
-  if (e == cudaSuccess) e = grow(k_box_axis<AXIS_FWD>, as);
-  if (e == cudaSuccess) e = grow(k_box_axis<AXIS_FGI>, as);
-  if (e == cudaSuccess) e = grow(k_box_axis<AXIS_INV>, as);
+  static SmemLimit row[2];
+  cudaError_t e = raise_smem(k_box_row<NM, false>, rs, row[0]);
+  if (e == cudaSuccess) e = raise_smem(k_box_row<NM, true>, rs, row[1]);
+  if (e == cudaSuccess) e = box_axis_smem(as);
   if (e != cudaSuccess) return e;
   const unsigned rows = (unsigned)(b.box.bn[1] * b.box.bn[2]);
   const unsigned cols = (unsigned)((b.Q - 1) * (b.NA / kBoxTx) + (b.xlast + kBoxTx - 1) / kBoxTx);

@@ -24,6 +24,7 @@
 #include <atomic>
 
 #include "mbo_dev.cuh"
+#include "mbo_limits.h"
 #include "mbo_select.cuh"
 
 namespace mbo {
@@ -804,31 +805,19 @@ cudaError_t launch_volume(VolumePass which, const Geom& g, const R* At, R* A, un
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-// Raise a kernel's dynamic shared-memory limit once (per process) to the
-// largest size it was launched with; launches inside graph capture then make
-// no attribute call.
-template <typename K> static cudaError_t set_smem(K kernel, size_t bytes, size_t& done) {
-  if (bytes <= 48 * 1024 || bytes <= done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) done = bytes;
-  return e;
-}
-
 // Blocks of a kernel that fit on the current device at once (at least one per
 // SM).  `last` keeps the last answer with its question (threads, shared bytes,
 // device) in one word, so that a loop of steps asks the runtime once.
 template <typename K>
 static int resident_blocks(K kernel, int threads, size_t smem, std::atomic<unsigned long long>& last) {
-  int dev = 0;
-  cudaGetDevice(&dev);
+  const int dev = current_device();
   const unsigned long long key = ((unsigned long long)(dev & 63) << 30 | (unsigned long long)threads << 20 |
                                   (unsigned long long)(smem >> 4 & 0xFFFFF)) << 20;
   const unsigned long long was = last.load(std::memory_order_relaxed);
   if ((was & ~0xFFFFFull) == key && (was & 0xFFFFF)) return (int)(was & 0xFFFFF);
-  int sms = 1, per_sm = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-  const int n = sms * (per_sm > 0 ? per_sm : 1);
+  const int n = device_sms(dev) * (per_sm > 0 ? per_sm : 1);
   last.store(key | (unsigned long long)n, std::memory_order_relaxed);
   return n;
 }
@@ -838,9 +827,9 @@ static cudaError_t launch_row_nm(const Geom& g, const Tables<R>& t, const R* Ain
                                  const StatsPtrs& sp, R fb, int threads, cudaStream_t s,
                                  bool prepare_only = false) {
   auto k = k_row<R, NM, MODE>;
-  static size_t done = 0;
+  static SmemLimit limit;  // raised once a device: launches inside graph capture make no attribute call
   const size_t smem = row_smem_bytes(g, sizeof(R), MODE == ROW_INV_PROJECT_FWD);
-  cudaError_t e = set_smem(k, smem, done);
+  cudaError_t e = raise_smem(k, smem, limit);
   if (e != cudaSuccess || prepare_only) return e;
   int rows = g.nz * g.ny;
   if (MODE == ROW_INV_PROJECT_FWD) {
@@ -881,10 +870,10 @@ static cudaError_t launch_axis_m(const Geom& g, const Tables<R>& t, void* W, con
                                  int axis, int tx, int threads, cudaStream_t s,
                                  bool prepare_only = false) {
   auto k = k_axis<R, MODE>;
-  static size_t done = 0;
+  static SmemLimit limit;  // raised once a device: launches inside graph capture make no attribute call
   const int L = axis == 1 ? g.ny : g.nz;
   const size_t smem = axis_smem_bytes(L, tx, sizeof(R));
-  cudaError_t e = set_smem(k, smem, done);
+  cudaError_t e = raise_smem(k, smem, limit);
   if (e != cudaSuccess || prepare_only) return e;
   int ltx = 0;
   while ((1 << ltx) < tx) ++ltx;

@@ -1084,11 +1084,11 @@ template <typename T, int CG> cudaError_t spread_run(const SpreadArgs<T>& a, dim
       return cudaGetLastError();
     }
   }
-  auto k = sizeof(T) == 8 && a.W == 7 ? k_spread<T, CG, sizeof(T) == 8 ? 7 : 0> : k_spread<T, CG, 0>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const bool w7 = sizeof(T) == 8 && a.W == 7;
+  auto k = w7 ? k_spread<T, CG, sizeof(T) == 8 ? 7 : 0> : k_spread<T, CG, 0>;
+  static SmemLimit limit[2];
+  const cudaError_t e = raise_smem(k, smem, limit[w7]);
+  if (e != cudaSuccess) return e;
   k<<<grid, kSpreadThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
@@ -1135,11 +1135,11 @@ template <typename T, int NM> cudaError_t interp_run(const InterpArgs<T>& a, int
       return cudaGetLastError();
     }
   }
-  auto k = a.W == 7 ? k_interp<T, NM, sizeof(T) == 4 && (NM == 2 || NM == 3) ? 0 : 7> : k_interp<T, NM, 0>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  constexpr int W7 = sizeof(T) == 4 && (NM == 2 || NM == 3) ? 0 : 7;
+  auto k = a.W == 7 ? k_interp<T, NM, W7> : k_interp<T, NM, 0>;
+  static SmemLimit limit[2];
+  const cudaError_t e = raise_smem(k, smem, limit[a.W == 7 && W7]);
+  if (e != cudaSuccess) return e;
   k<<<groups, kInterpBlock, smem, st>>>(a);
   return cudaGetLastError();
 }

@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "mbo_limits.h"
+
 namespace mbo {
 
 // Length N = R * M with M in {256, 512, 1024} and R in {1, 2, 3} (see WarpFFTR).
@@ -67,13 +69,6 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), int blocks, int threads, siz
   cfg.attrs = at;
   cfg.numAttrs = pdl_flag() ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
-}
-
-template <typename K> inline cudaError_t set_smem_once(K kernel, size_t bytes, size_t& done) {
-  if (bytes <= 48 * 1024 || bytes <= done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) done = bytes;
-  return e;
 }
 
 }  // namespace mbo
