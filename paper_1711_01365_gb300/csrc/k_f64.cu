@@ -6,10 +6,10 @@ namespace mbo {
 
 namespace {
 
-template <int NM, int MODE>
-cudaError_t row_fx(const Geom& g, const Tables<double>& t, const double* Ain, double* A, void* W,
+template <int NM, int MODE, bool SHORT>
+cudaError_t row_fx_form(const Geom& g, const Tables<double>& t, const double* Ain, double* A, void* W,
                    const StatsPtrs& sp, int threads, cudaStream_t s, bool prepare_only = false) {
-  auto k = k_row_fx<NM, MODE>;
+  auto k = k_row_fx<NM, MODE, SHORT>;
   static SmemLimit limit;
   const size_t smem = row_smem_bytes(g, sizeof(double), false);
   const cudaError_t e = raise_smem(k, smem, limit);
@@ -21,6 +21,13 @@ cudaError_t row_fx(const Geom& g, const Tables<double>& t, const double* Ain, do
   }
   k<<<rows, threads, smem, s>>>(g, t, Ain, A, static_cast<double2*>(W), sp);
   return cudaGetLastError();
+}
+
+template <int NM, int MODE>
+cudaError_t row_fx(const Geom& g, const Tables<double>& t, const double* Ain, double* A, void* W,
+                   const StatsPtrs& sp, int threads, cudaStream_t s, bool prepare_only = false) {
+  if (fx_short_rows(g)) return row_fx_form<NM, MODE, true>(g, t, Ain, A, W, sp, threads, s, prepare_only);
+  return row_fx_form<NM, MODE, false>(g, t, Ain, A, W, sp, threads, s, prepare_only);
 }
 
 template <int NM>

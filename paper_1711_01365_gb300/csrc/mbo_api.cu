@@ -130,6 +130,11 @@ Plan make_plan(int N, PlanFor want) {
 // time.  FP64: 128^2, n = 2: y pass 29 -> 23 us, x pass 31 -> 23 us.
 constexpr long long kSmall64 = 1500000, kSmall32 = 300000;
 
+PlanFor plan_for(const Geom& g, bool f32) {
+  if (g.P * g.Q > (f32 ? kSmall32 : kSmall64)) return PlanFor::kThroughput;
+  return f32 ? PlanFor::kSmall32 : PlanFor::kSmall64;
+}
+
 Plan axis_plan(const Geom& g, int axis, bool f32) {
   const int N = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
   if (f32 && warp_plan_length(N) && (axis == 0 || warp_tile(N, g.nx, 8) != 0) &&
@@ -140,8 +145,7 @@ Plan axis_plan(const Geom& g, int axis, bool f32) {
     p.lq = N / p.rad0 == 1024 ? 32 : 16;
     return p;
   }
-  if (g.P * g.Q > (f32 ? kSmall32 : kSmall64)) return make_plan(N);
-  return make_plan(N, f32 ? PlanFor::kSmall32 : PlanFor::kSmall64);
+  return make_plan(N, plan_for(g, f32));
 }
 
 int plan_twiddles(const Plan& p) {
@@ -177,6 +181,12 @@ int pick_tx(int nx, int cap) {
   int t = 1;
   while (t < cap && nx % (2 * t) == 0) t *= 2;
   return t;
+}
+
+int fx_row_threads(const Geom& g) {
+  if (fx_short_rows(g)) return std::min(kMaxThreads, (g.nx + 31) / 32 * 32 * g.Q);
+  if (row_smem_bytes(g, 8, false) > 114 * 1024) return 384;
+  return g.nx >= 256 ? 192 : g.nx >= 64 ? 128 : (g.nx + 31) / 32 * 32;
 }
 
 int net_tile(int nx, int cap) {
@@ -861,11 +871,12 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
   // for long rows of several planes (1296 points, n = 3: 192 threads 110 us, 256
   // threads 103).  FP64 rows (168 registers: 384 threads fit on an SM): 192 from
   // 256 points on, 384 where a row fills the SM's shared memory, 128 for short
-  // rows (128^2, n = 2: 64 threads 26.6 us, 128 threads 23.1 us).
+  // rows (128^2, n = 2: 64 threads 26.6 us, 128 threads 23.1 us), a thread per point
+  // below 64 (48^3, n = 3: 32 threads 216 us a step, 64 threads 210, 128 threads 247).
   if (dtype == MBO_F32)
     h->row_threads = g.nx <= 192 ? std::max(32, (g.nx + 31) / 32 * 32) : g.nx >= 1200 && n >= 3 ? 256 : 192;
   else
-    h->row_threads = row_smem_bytes(g, 8, false) > 114 * 1024 ? 384 : g.nx >= 256 ? 192 : g.nx >= 64 ? 128 : 32;
+    h->row_threads = fx_row_threads(g);
   // Strided passes: as many threads as a stage of the longest network axis has
   // butterflies (tiles of 96 x 8, n = 3, 96^3: 256 threads 78 us, 64 threads 37.5;
   // 486 x 8: 64 threads 31.1 us, 256 threads 23.3), 256 at most in FP32 and 128 in
@@ -875,7 +886,7 @@ mbo_status mbo_create(mbo_handle* out, int ndim, const int64_t* dims, int n, dou
   for (int ax = 1; ax < ndim; ++ax)
     if (!axis_plan(g, ax, dtype == MBO_F32).lq) longest = std::max(longest, ax == 1 ? g.ny : g.nz);
   if (dtype == MBO_F32) h->axis_threads = longest <= 96 ? 64 : longest <= 192 ? 128 : longest <= 288 ? 192 : 256;
-  else h->axis_threads = longest <= 96 ? 64 : 128;
+  else h->axis_threads = fx_axis_threads(longest);
   if (dtype == MBO_F32) {
     // FP32 warp-plan strided passes, measured on GB300: 16-column tiles (one
     // 128-byte line per tile row) where an axis of 512 is strided (512^3:

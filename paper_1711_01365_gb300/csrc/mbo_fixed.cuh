@@ -401,7 +401,13 @@ template <class Each> __device__ FxScale fx_scale_slow(Each each, int r, unsigne
 // |z| <= sqrt(2) and the sum of N of them stays below 2^(ceil(log2 N) + 1/2).
 __device__ __forceinline__ int fx_unit_scale(int N) { return 61 - (32 - __clz(N - 1)); }
 
-template <int NM, int MODE>
+// SHORT: the form for few rows of at most 64 points.  There a block's own chain of
+// instructions is the time (32^2, n = 3: 2800 a warp, one after another in the one
+// warp that a row has points for, each fetched for the first time), so the planes
+// are spread over groups of warps, and each group runs one copy of a plane's
+// conversions.  Long rows unroll the planes instead: their conversions overlap
+// (96^3, n = 3, diffusion: 831 us, 892 with the planes in turn).
+template <int NM, int MODE, bool SHORT>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, double2* W, StatsPtrs sp) {
   constexpr int C = NM * NM, Q = (C + 1) / 2;
@@ -410,6 +416,7 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
   __shared__ StatsShared<double, MODE == ROW_INV_PROJECT_FWD ? kMaxThreads : 1> sh;
   __shared__ float rs[2][12][Q];
   __shared__ int drops[Q];
+  __shared__ int ks[Q], kins[Q];  // scale exponents of the planes whose norm is out of the FP32 range (SHORT: all)
   __shared__ unsigned slow[32];
   __shared__ int s_flag, s_bad;
   if (sp.respect_stop && *(volatile int*)&sp.st->stop) return;
@@ -421,19 +428,113 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
   const long long P = g.P;
   const int T = blockDim.x, tid = threadIdx.x;
   const FxTw* tw = static_cast<const FxTw*>(t.tw[0]);
-  int k[Q];  // scale exponent of each plane's sequence
+  // scale exponent of each plane's sequence (SHORT: in ks), less the lift of the planes in `lifted`
+  int k[Q] = {};
+  unsigned lifted = 0;
+  // SHORT: group `grp` of `ng` groups of `gthreads` threads takes planes grp, grp + ng, ...;
+  // threads past the last group take none
+  const int wpp = (nx + 31) >> 5, ng = SHORT ? max(1, min(Q, (T >> 5) / wpp)) : 1;
+  const int gthreads = SHORT ? (ng == 1 ? T : wpp << 5) : T;
+  const int grp = SHORT ? tid / gthreads : 0, gt = tid - grp * gthreads;
+  // f(q, x) over this thread's share of the planes' entries
+  auto visit = [&](auto f) {
+    if constexpr (SHORT) {
+      if (grp < ng) {
+#pragma unroll 1
+        for (int q = grp; q < Q; q += ng)
+          for (int x = gt; x < nx; x += gthreads) f(q, x);
+      }
+    } else {
+      for (int x = tid; x < nx; x += T) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) f(q, x);
+      }
+    }
+  };
+  auto scale_of = [&](int q) {
+    if constexpr (SHORT) return ks[q];
+    else return k[q];
+  };
 
   // scales of the Q sequences in sd, and the sequences converted in place, for
   // a transform whose first stage has radix r (inverse: parts swapped)
-  auto to_fixed = [&](int r, bool swap) {
+  // The slow scales of the planes in `todo` (all threads call it; it ends in a barrier).
+  auto slow_scales = [&](unsigned todo, int r) {
+#pragma unroll 1
+    for (int q = 0; q < Q; ++q) {
+      if (!(todo >> q & 1)) continue;
+      auto points = [&](auto each) {
+        for (int x = tid; x < nx; x += T) each(sd[lay.addr(q, x)]);
+      };
+      const FxScale f = fx_scale_slow(points, r, slow);
+      const int up = fx_lift(f.in), down = fx_lift(f.k);
+      if (up) points([](double2& z) { fx_scale2(z, 0x1p600); });
+      if (down) lifted |= 1u << q;
+      if (tid == 0) {
+        ks[q] = f.k == kFxBad ? kFxBad : f.k - down;
+        kins[q] = f.in - up;
+        drops[q] = f.k == kFxBad ? 0 : f.in - f.k;
+      }
+    }
+    __syncthreads();
+  };
+  auto to_fixed_short = [&](int r, bool swap) {
+    const int gw = gthreads >> 5;  // warps of a group
+    if (grp < ng) {
+#pragma unroll 1
+      for (int q = grp; q < Q; q += ng) {
+        float n = 0.f, mx = 0.f;
+        for (int x = gt; x < nx; x += gthreads) {
+          const float a = fx_norm(sd[lay.addr(q, x)]);
+          n += a;
+          mx = fmaxf(mx, a);
+        }
+        n = warp_sum(n);
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+        if ((tid & 31) == 0) {
+          rs[0][gt >> 5][q] = n;
+          rs[1][gt >> 5][q] = __uint_as_float(m);
+        }
+      }
+    }
+    __syncthreads();
+    // the scales, a thread per plane
+    bool plain = true;
+    if (tid < Q) {
+      float sum = 0.f, top = 0.f;
+      for (int w = 0; w < gw; ++w) {
+        sum += rs[0][w][tid];
+        top = fmaxf(top, rs[1][w][tid]);
+      }
+      plain = fx_plain(sum);
+      const FxScale f = plain ? fx_scales(sum, top, 0, r) : FxScale{0, 0};
+      ks[tid] = f.k;
+      kins[tid] = f.in;
+      drops[tid] = f.in - f.k;
+      slow[tid] = plain ? 0u : 1u;
+    }
+    lifted = 0;
+    if (!__syncthreads_and(plain)) {
+      unsigned todo = 0;
+      for (int q = 0; q < Q; ++q) todo |= slow[q] << q;
+      slow_scales(todo, r);
+    }
+    visit([&](int q, int x) {
+      const int a = lay.addr(q, x), kin = kins[q];
+      const double2 z = sd[a];
+      const long long re = fx_from(z.x, kin), im = fx_from(z.y, kin);
+      s[a] = ks[q] == kFxBad ? fx2{0, 0} : swap ? fx2{im, re} : fx2{re, im};
+    });
+    __syncthreads();
+  };
+  auto to_fixed_long = [&](int r, bool swap) {
     float n[Q], mx[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) n[q] = mx[q] = 0.f;
     for (int x = tid; x < nx; x += T) {
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        const double2 z = sd[lay.addr(q, x)];
-        const float a = fx_norm(z);
+        const float a = fx_norm(sd[lay.addr(q, x)]);
         n[q] += a;
         mx[q] = fmaxf(mx[q], a);
       }
@@ -449,6 +550,7 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
     }
     __syncthreads();
     int kin[Q];
+    unsigned todo = 0;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       float sum = 0.f, top = 0.f;
@@ -456,21 +558,22 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
         sum += rs[0][w][q];
         top = fmaxf(top, rs[1][w][q]);
       }
-      FxScale f;
-      int up = 0;
-      if (fx_plain(sum)) {
-        f = fx_scales(sum, top, 0, r);
-      } else {
-        auto points = [&](auto each) {
-          for (int x = tid; x < nx; x += T) each(sd[lay.addr(q, x)]);
-        };
-        f = fx_scale_slow(points, r, slow);
-        up = fx_lift(f.in);
-        if (up) points([](double2& z) { fx_scale2(z, 0x1p600); });
-      }
+      const bool plain = fx_plain(sum);  // the same in every thread
+      const FxScale f = plain ? fx_scales(sum, top, 0, r) : FxScale{0, 0};
+      todo |= plain ? 0u : 1u << q;
       k[q] = f.k;
-      kin[q] = f.in - up;
-      if (tid == 0) drops[q] = f.k == kFxBad ? 0 : f.in - f.k;
+      kin[q] = f.in;
+      if (tid == 0) drops[q] = f.in - f.k;
+    }
+    lifted = 0;
+    if (todo) {
+      slow_scales(todo, r);
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        if (todo >> q & 1) {
+          k[q] = ks[q];
+          kin[q] = kins[q];
+        }
     }
     for (int x = tid; x < nx; x += T) {
 #pragma unroll
@@ -482,6 +585,10 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
       }
     }
     __syncthreads();
+  };
+  auto to_fixed = [&](int r, bool swap) {
+    if constexpr (SHORT) to_fixed_short(r, swap);
+    else to_fixed_long(r, swap);
   };
   auto from_fixed = [&](fx2 v, int kk) {
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
@@ -505,14 +612,12 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
     __syncthreads();
     to_fixed(t.plan[0].st[0].rad, false);
     fft_fx(s, lay, nx, Q, t.plan[0], tw, false, drops);
-    for (int x = tid; x < nx; x += T) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) W[q * P + off + x] = from_fixed(s[lay.addr(q, x)], k[q] - fx_lift(k[q]));
+    visit([&](int q, int x) { W[q * P + off + x] = from_fixed(s[lay.addr(q, x)], scale_of(q)); });
+    if (lifted) {
+      visit([&](int q, int x) {
+        if (lifted >> q & 1) fx_scale2(W[q * P + off + x], 0x1p-600);
+      });
     }
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-      if (fx_lift(k[q]))
-        for (int x = tid; x < nx; x += T) fx_scale2(W[q * P + off + x], 0x1p-600);
     if (sp.do_stats) {
       const double tot = block_sum(defect, redd);
       double all;
@@ -535,14 +640,17 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
     fft_fx(s, lay, nx, Q, t.plan[0], tw, true, drops);
 
     if (MODE == ROW_INV_OUT) {
-      for (int x = tid; x < nx; x += T) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          double2 z = from_fixed(s[lay.addr(q, x)], k[q] - fx_lift(k[q]));  // swapped
-          if (fx_lift(k[q])) fx_scale2(z, 0x1p-600);
-          A[(2 * q) * P + off + x] = z.y;
-          if (2 * q + 1 < C) A[(2 * q + 1) * P + off + x] = z.x;
-        }
+      visit([&](int q, int x) {
+        const double2 z = from_fixed(s[lay.addr(q, x)], scale_of(q));  // swapped
+        A[(2 * q) * P + off + x] = z.y;
+        if (2 * q + 1 < C) A[(2 * q + 1) * P + off + x] = z.x;
+      });
+      if (lifted) {
+        visit([&](int q, int x) {
+          if (!(lifted >> q & 1)) return;
+          A[(2 * q) * P + off + x] *= 0x1p-600;
+          if (2 * q + 1 < C) A[(2 * q + 1) * P + off + x] *= 0x1p-600;
+        });
       }
       return;
     }
@@ -553,12 +661,17 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
     const int ku = fx_unit_scale(nx);
     const int kin = t.plan[0].nst > 1 ? 61 - (32 - __clz(t.plan[0].st[0].rad - 1)) : ku;
     int bad = 0;
-    {  // the polar factor does not depend on the scale: where every plane is lifted, m stays so
-      int up = kFxUp;
+    // the polar factor does not depend on the scale: where every plane is lifted or zero, m
+    // stays so
+    bool all = true;
 #pragma unroll
-      for (int q = 0; q < Q; ++q) up = min(up, fx_lift(k[q]));
+    for (int q = 0; q < Q; ++q) {
+      k[q] = scale_of(q);
+      all = all && ((lifted >> q & 1) || k[q] == 0);
+    }
+    if (!all) {
 #pragma unroll
-      for (int q = 0; q < Q; ++q) k[q] -= up;
+      for (int q = 0; q < Q; ++q) k[q] += lifted >> q & 1 ? kFxUp : 0;
     }
     for (int x = tid; x < nx; x += T) {
       double old[C], m[C], b[C], sg;
@@ -592,11 +705,9 @@ k_row_fx(Geom g, Tables<double> t, const double* __restrict__ Ain, double* A, do
     const int planes_bad = s_bad;
     if (end && sp.do_stats) last = stats_arrive(sp, sh);
     fft_fx(s, lay, nx, Q, t.plan[0], tw, false, drops);
-    for (int x = tid; x < nx; x += T) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q)
-        W[q * P + off + x] = from_fixed(s[lay.addr(q, x)], (planes_bad >> q & 1) ? kFxBad : ku);
-    }
+    visit([&](int q, int x) {
+      W[q * P + off + x] = from_fixed(s[lay.addr(q, x)], (planes_bad >> q & 1) ? kFxBad : ku);
+    });
     if (end) break;
     __syncthreads();  // the row is in W: its slots are free
   }

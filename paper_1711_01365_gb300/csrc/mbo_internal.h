@@ -228,6 +228,7 @@ FastDiv make_div(unsigned d);
 // FP32 or a fixed-point pass.
 enum class PlanFor { kThroughput, kSmall32, kSmall64 };
 Plan make_plan(int N, PlanFor want = PlanFor::kThroughput);
+PlanFor plan_for(const Geom& g, bool f32);  // what the network plans of a geometry are chosen for
 // Plan of one axis of a geometry: the warp-cooperative plan (FP32, lengths
 // 256, 512, 768, 1024, 1536, 2048; strided axes need nx % 4 == 0) where one
 // exists, else make_plan.
@@ -236,6 +237,13 @@ int plan_twiddles(const Plan& p);
 // pos[k]: position where the forward transform of a plan leaves frequency k.
 void digit_positions(const Plan& p, int N, std::vector<int>& pos);
 int pick_tx(int nx, int cap);
+// Rows of the FP64 x pass that take its form for few short rows (k_row_fx), and the
+// threads of its blocks: a block per SM at most, so that each may take a warp per
+// plane and 32 points (32^2, n = 3, diffusion: 41.0 -> 32.8 us).
+inline bool fx_short_rows(const Geom& g) { return g.nx <= 64 && (long long)g.ny * g.nz <= 152; }
+int fx_row_threads(const Geom& g);
+// Threads of the FP64 strided passes over axes of up to `longest` points.
+inline int fx_axis_threads(int longest) { return longest <= 96 ? 64 : 128; }
 // Columns per tile of the network strided passes: `cap` (64 bytes a tile row),
 // or the power of two that covers a narrower field.
 int net_tile(int nx, int cap);

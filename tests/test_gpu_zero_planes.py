@@ -66,3 +66,19 @@ def test_zero_columns_beside_live_ones(M, dims, scale):
     h.close()
     lim = 3e-15 * float(want.abs().max())
     assert float((out / scale - want).abs().max()) <= lim
+
+
+@pytest.mark.parametrize("dims,n", [((16, 16), 3), ((96, 128), 3), ((96, 128), 2)])
+def test_step_of_subnormal_phases(M, dims, n):
+    """The projection does not depend on the scale: two constant phases times 2^-1030,
+    most channels zero, step like the phases themselves."""
+    A = torch.zeros((n * n,) + dims, device="cuda", dtype=torch.float64)
+    for i in range(n):
+        A[i * n + i] = 1.0
+    A[0, ..., : dims[-1] // 2] = -1.0
+    B = A * 2.0 ** -600 * 2.0 ** -430
+    h = M.Mbo(dims, n, 3.0 / min(dims) ** 2, "f64")
+    h.step(A)
+    h.step(B)
+    h.close()
+    assert float((A - B).abs().max()) <= 1e-9
