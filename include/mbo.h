@@ -116,9 +116,11 @@ MBO_API void mbo_default_config(mbo_config* cfg);
 
 /* The launch shapes a handle uses (after any autotuning): row_threads,
  * axis_threads, axis_tx, axis_stages and pdl (1 on, 2 off) filled in; the
- * other fields as the handle was created with.  (Where axis_tx was automatic,
- * axes without a warp plan may take tiles of another width than it reports:
- * full ones with a ragged last tile, or narrower ones for small fields.) */
+ * other fields as the handle was created with.  A handle created with these
+ * values takes the same launch shapes.  (Axes without a warp plan may take tiles
+ * of another width than axis_tx reports: full ones with a ragged last tile where
+ * only the width of the field would force narrower ones, and, beside an axis with a
+ * warp plan, narrower ones for small fields.) */
 MBO_API mbo_status mbo_launch_config(mbo_handle h, mbo_config* out);
 
 /* Create a handle for one field geometry.

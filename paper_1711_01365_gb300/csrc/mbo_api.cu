@@ -600,7 +600,8 @@ template <typename R> __global__ void k_tune_fill(R* A, long long n) {
 }
 
 // Columns per tile of the handle's network strided passes where the tile width
-// setting is tx: an explicit width as it is; else a narrow one, which only the
+// setting is tx: an explicit width as it is, unless it is what only the field's width
+// forces (and mbo_launch_config reports for ragged tiles); else a narrow one, which only the
 // field's width forces (tx divides nx), gives way to a full tile with a ragged
 // last one (64 bytes of each row instead of 16 for nx = 486, 8 for nx = 243), and
 // a field with fewer tiles than SMs takes narrower ones (128^2, n = 2, FP64 y
@@ -608,7 +609,7 @@ template <typename R> __global__ void k_tune_fill(R* A, long long n) {
 int net_width(const mbo_ctx* h, int tx) {
   const bool f32 = h->dtype == MBO_F32;
   const int cap = f32 ? 8 : 4;
-  if (h->cfg.axis_tx) return tx;
+  if (h->cfg.axis_tx && (h->cfg.axis_tx >= cap || h->cfg.axis_tx != pick_tx(h->g.nx, cap))) return tx;
   int w = tx >= cap ? tx : net_tile(h->g.nx, cap);
   const int outer = h->g.ndim == 3 ? std::min(h->g.ny, h->g.nz) : 1;
   while (w > (f32 ? 2 : 1) && (long long)h->g.Q * outer * ((h->g.nx + w - 1) / w) < 152) w /= 2;
@@ -702,8 +703,10 @@ mbo_status autotune(mbo_ctx* h, int maxsm) {
     if (t >= 1 && t <= 16 && std::find(txs.begin(), txs.end(), t) == txs.end()) txs.push_back(t);
   if (c.axis_tx) txs = {h->tx};
   stages = (warp_axis && !c.axis_stages) ? std::vector<int>{1, 2, 3} : std::vector<int>{h->axis_stages};
-  athreads = (net_axis && !c.axis_threads) ? std::vector<int>{128, 256, 384}
-                                           : std::vector<int>{h->axis_threads};
+  athreads = {h->axis_threads};  // the default is always a candidate
+  if (net_axis && !c.axis_threads)
+    for (int t : {128, 256, 384})
+      if (t != h->axis_threads) athreads.push_back(t);
   rthreads = (net_row && !c.row_threads) ? std::vector<int>{64, 128, 192, 256, 384}
                                          : std::vector<int>{h->row_threads};
   const size_t fbytes = (size_t)g.C * (size_t)g.P * h->elem;
@@ -1064,7 +1067,12 @@ mbo_status mbo_launch_config(mbo_handle h, mbo_config* out) {
   *out = h->cfg;
   out->row_threads = h->row_threads;
   out->axis_threads = h->axis_threads;
-  out->axis_tx = h->tx;
+  // the network passes' own width where they are the only strided ones and it may be given
+  // back (it divides nx)
+  bool warp = false;
+  for (int ax = 1; ax < h->g.ndim; ++ax) warp = warp || (h->dtype == MBO_F32 && h->tf.plan[ax].lq);
+  const int w = net_width(h, h->tx);
+  out->axis_tx = !warp && h->g.nx % w == 0 ? w : h->tx;
   out->axis_stages = h->axis_stages;
   out->pdl = h->pdl ? 1 : 2;
   return MBO_OK;
