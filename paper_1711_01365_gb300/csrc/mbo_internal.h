@@ -279,7 +279,7 @@ cudaError_t launch_volume(VolumePass which, const Geom& g, const R* At, R* A, un
                           SelectState* ss, const StatsPtrs& sp, double fb, int blocks,
                           cudaStream_t s, long long n_plus = 0);
 
-// Replace the per-axis multipliers of a handle's diffusion (mbo_api.cu).
+// Replace the per-axis multipliers of an FP64 handle's diffusion (mbo_api.cu).
 // mult[ax] (ax = 0: x, 1: y, 2: z; z ignored in 2-D) holds N_ax values in
 // natural frequency order: index k is the signed frequency k (2k <= N) or
 // k - N.  The diffusion then multiplies spectrum entry (kz, ky, kx) by

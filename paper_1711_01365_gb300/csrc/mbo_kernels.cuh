@@ -1,6 +1,7 @@
 // Kernels of the flat-torus MBO step (Algorithm 1 of Osting & Wang,
-// arXiv:1711.01365) and their launchers.  Instantiated per element type in
-// k_f32.cu and k_f64.cu.
+// arXiv:1711.01365) and their launchers.  The passes over rows and columns here
+// are those of FP32 fields on axes without a warp plan (k_f32.cu; FP64:
+// mbo_fixed.cuh); the pointwise kernels are instantiated for both types.
 //
 // Data layout in HBM
 //   field A      planar: channel c = i*n + j, P values each, row-major (z, y, x)
@@ -369,7 +370,7 @@ __device__ __forceinline__ void stats_finish(long long P, double tau, const Stat
 }
 
 template <typename R, int NM, int MODE>
-__global__ void __launch_bounds__(kMaxThreads, sizeof(R) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(kMaxThreads, 2)
 k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W, StatsPtrs sp,
       R fb_sigma) {
   using V = typename VT<R>::V;
@@ -388,7 +389,6 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
   long long off = (long long)blockIdx.x * nx;
   const int T = blockDim.x, tid = threadIdx.x;
   const V* tw = static_cast<const V*>(t.tw[0]);
-  const bool is_f32 = sizeof(R) == 4;
 
   if (MODE == ROW_FWD) {
     R defect = R(0);
@@ -477,7 +477,7 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
     }
     finish_point<NM>(A, P, off, x, old, b, sg, s + lay.addr(0, x), lay.S, ps);
   }
-  if (is_f32 && NM >= 2) {
+  if (NM >= 2) {
     __syncthreads();
     const int nf = min(s_nfb, kFallbackCap);
     for (int k = tid; k < nf; k += T) {
@@ -513,7 +513,7 @@ k_row(Geom g, Tables<R> t, const R* __restrict__ Ain, R* A, typename VT<R>::V* W
 // Strided-axis pass (y in 2-D; y and z in 3-D).  One block owns a tile of tx
 // adjacent x-columns of one complex plane along the whole axis.
 template <typename R, int MODE>
-__global__ void __launch_bounds__(kMaxThreads, sizeof(R) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(kMaxThreads, 2)
 k_axis(Geom g, Tables<R> t, typename VT<R>::V* W, StatsPtrs sp, int axis, int ltx) {
   using V = typename VT<R>::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -844,9 +844,7 @@ template <typename R>
 cudaError_t launch_row(RowMode mode, const Geom& g, const Tables<R>& t, const R* A_in, R* A_out,
                        void* W, const StatsPtrs& sp, double fallback_sigma, int threads,
                        cudaStream_t s) {
-  if constexpr (sizeof(R) == 4) {
-    if (t.plan[0].lq) return launch_wrow(mode, g, t, A_in, A_out, W, sp, fallback_sigma, s, false);
-  }
+  if (t.plan[0].lq) return launch_wrow(mode, g, t, A_in, A_out, W, sp, fallback_sigma, s, false);
   const R fb = (R)fallback_sigma;
 #define MBO_ROW_CASE(NM)                                                                   \
   if (g.n == NM) {                                                                         \
@@ -888,10 +886,8 @@ cudaError_t launch_axis(AxisMode mode, int axis, const Geom& g, const Tables<R>&
                         const StatsPtrs& sp, int tx, int threads, cudaStream_t s,
                         const CUtensorMap* tm, int stages, const void* l2_hint,
                         long long l2_hint_bytes) {
-  if constexpr (sizeof(R) == 4) {
-    if (t.plan[axis].lq)
-      return launch_wcol(mode, axis, g, t, W, sp, tx, s, false, tm, stages, l2_hint, l2_hint_bytes);
-  }
+  if (t.plan[axis].lq)
+    return launch_wcol(mode, axis, g, t, W, sp, tx, s, false, tm, stages, l2_hint, l2_hint_bytes);
   switch (mode) {
     case AXIS_FWD: return launch_axis_m<R, AXIS_FWD>(g, t, W, sp, axis, tx, threads, s);
     case AXIS_INV: return launch_axis_m<R, AXIS_INV>(g, t, W, sp, axis, tx, threads, s);
@@ -922,16 +918,14 @@ template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>
   Tables<R> t{};
   StatsPtrs sp{};
   cudaError_t e = cudaSuccess;
-  if constexpr (sizeof(R) == 4) {
-    if (tabs.plan[0].lq) {
-      for (int m = ROW_FWD; m <= ROW_INV_PROJECT_FWD && e == cudaSuccess; ++m)
-        e = launch_wrow((RowMode)m, g, tabs, nullptr, nullptr, nullptr, sp, 0.0, 0, true);
-    }
-    for (int axis = 1; axis <= (g.ndim == 3 ? 2 : 1) && e == cudaSuccess; ++axis) {
-      if (!tabs.plan[axis].lq) continue;
-      for (int m = AXIS_FWD; m <= AXIS_ENERGY && e == cudaSuccess; ++m)
-        e = launch_wcol((AxisMode)m, axis, g, tabs, nullptr, sp, tx, 0, true, nullptr, stages);
-    }
+  if (tabs.plan[0].lq) {
+    for (int m = ROW_FWD; m <= ROW_INV_PROJECT_FWD && e == cudaSuccess; ++m)
+      e = launch_wrow((RowMode)m, g, tabs, nullptr, nullptr, nullptr, sp, 0.0, 0, true);
+  }
+  for (int axis = 1; axis <= (g.ndim == 3 ? 2 : 1) && e == cudaSuccess; ++axis) {
+    if (!tabs.plan[axis].lq) continue;
+    for (int m = AXIS_FWD; m <= AXIS_ENERGY && e == cudaSuccess; ++m)
+      e = launch_wcol((AxisMode)m, axis, g, tabs, nullptr, sp, tx, 0, true, nullptr, stages);
   }
 #define MBO_PREP_ROW(NM)                                                                       \
   if (g.n == NM) {                                                                             \
@@ -950,7 +944,7 @@ template <typename R> cudaError_t prepare_kernels(const Geom& g, const Tables<R>
   MBO_PREP_ROW(4)
 #undef MBO_PREP_ROW
   for (int axis = 1; axis <= (g.ndim == 3 ? 2 : 1) && e == cudaSuccess; ++axis) {
-    if (sizeof(R) == 4 && tabs.plan[axis].lq) continue;  // the warp-plan pass above takes this axis
+    if (tabs.plan[axis].lq) continue;  // the warp-plan pass above takes this axis
     e = launch_axis_m<R, AXIS_FWD>(g, t, nullptr, sp, axis, net_tx, 64, 0, true);
     if (e == cudaSuccess) e = launch_axis_m<R, AXIS_INV>(g, t, nullptr, sp, axis, net_tx, 64, 0, true);
     if (e == cudaSuccess) e = launch_axis_m<R, AXIS_FGI>(g, t, nullptr, sp, axis, net_tx, 64, 0, true);

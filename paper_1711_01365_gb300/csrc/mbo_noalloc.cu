@@ -60,7 +60,10 @@ __global__ void k_noalloc_tables(Plan pl, int N, int ntw, double tau, typename V
           const long long e = ((long long)n1 * j) % s.lb;
           double sn, cs;
           sincospi(2.0 * (double)e / (double)s.lb, &sn, &cs);
-          if constexpr (sizeof(R) == 8) {  // Q60 limbs of the fixed-point transforms
+          if constexpr (sizeof(R) == 8) {
+            // Q60 limbs of the fixed-point transforms, from FP64 values: 53 bits of the 60 that a
+            // handle's tables have (128^2, n = 3: RMS error of the diffusion 5.0e-17, a handle's
+            // 4.2e-17, FP64 transforms' 1.5e-16)
             *reinterpret_cast<FxTw*>(&tw[i]) =
                 fx_tw(__double2ll_rn(cs * 0x1p60), __double2ll_rn(-sn * 0x1p60));
           } else {

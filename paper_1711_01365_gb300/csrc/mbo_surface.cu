@@ -104,9 +104,9 @@ template <typename T> struct SpreadArgs {
 // WT: the kernel width as a compile-time constant (the width of eps = 1e-6,
 // the paper's choice, has its own instantiation), or 0 for the runtime width.
 template <typename T> __host__ __device__ constexpr int chunk_of() { return sizeof(T) == 4 ? 32 : 16; }
-// Tile column of x in tile row y.  At width 7 the rows are 16 wide and a flush
-// writes 4 rows x 8 columns from an even (x, y) start: x ^ 8 on rows with bit 1
-// of y set puts those 32 lanes on 32 distinct banks.
+// Tile column of x in tile row y.  At width 7 (FP64 only: FP32 has k_spread7) the rows
+// are 16 wide, 128 bytes: x ^ 8 on rows with bit 1 of y set spreads the 4 rows x 8
+// columns that a flush writes over the banks.
 template <int WT> __device__ __forceinline__ int swz(int x, int y) {
   if constexpr (WT == 7) return x ^ (((y >> 1) & 1) << 3);
   return x;
