@@ -1100,10 +1100,12 @@ static __device__ __noinline__ double polar4_jacobi(const double* m, double* b, 
 //   Last step.  After an unscaled step every singular value is 1 + d, d >= 0, so
 // e = |det X| - 1 bounds the d: at kNewtonLast the next step ends at d^2 / 2 below
 // 2e-17.  1 / |det X| is 1 - e + e^2 to e^3.
-// Taken where FP32 holds m and its class is clear: |det m| above
-// kNewtonDet |m|^3 (the smallest singular value is then above 1e-4 |m|, which FP32
-// resolves); elsewhere false, and the caller goes on with polar_newton.
-constexpr float kNewtonDet = 1e-4f;
+// Taken where FP32 holds m and its class is clear: |det m| above kNewtonDet |m|^3,
+// a hundred times the rounding of the FP32 determinant (and the smallest singular
+// value is then above 1e-5 |m|, known to 1%, enough for coefficients); elsewhere
+// false, and the caller goes on with polar_newton.  At 1e-4 1 random matrix in 700
+// was left, and a warp waits for the iteration of any.
+constexpr float kNewtonDet = 1e-5f;
 constexpr float kNewtonNear = 1.5e-4f;  // sum of s^2 - 1 that ends the scaled steps
 constexpr double kNewtonLast = 6e-9;
 
@@ -1113,11 +1115,21 @@ __device__ __forceinline__ double half_bits(double x) {
   return __hiloint2double((hi & 0x7ff00000) ? hi - 0x00100000 : hi, __double2loint(x));
 }
 
+// x in FP32, cut off instead of rounded, in the integer pipe (a conversion holds the
+// FP64 pipe like an addition); 0 and infinity beyond FP32's normal range
+__device__ __forceinline__ float float_bits(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), t = hi & 0x7fffffffu;
+  // exponent and mantissa shifted to their place, the exponent's offset moved by 1023 - 127
+  unsigned f = __funnelshift_l((unsigned)__double2loint(x), hi, 3) + 0x40000000u;
+  f = t < 0x38100000u ? 0u : t >= 0x47f00000u ? 0x7f800000u : f;
+  return __uint_as_float(f | (hi & 0x80000000u));
+}
+
 __device__ __forceinline__ bool polar3_guided(const double* m, double* b, double& sg) {
   float x[9], c[9], nx = 0.f;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    x[k] = (float)m[k];
+    x[k] = float_bits(m[k]);
     nx += x[k] * x[k];
   }
   if (!(nx > 1e-24f && nx < 1e24f)) return false;  // out of range, or not finite
