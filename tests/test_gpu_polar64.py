@@ -77,3 +77,27 @@ def test_projection_error(M, kind, scale, fused):
     assert defect.max() <= 8e-16 and defect.mean() <= 1.6e-16
     if RMS[kind]:
         assert np.sqrt((err ** 2).mean()) <= RMS[kind]
+
+
+@pytest.mark.parametrize("dims", [(48, 64), (72, 72, 96), (512, 96)])
+def test_step_statistics_equal_the_unfused_ones(M, dims):
+    """n = 3: the fused step's field and records against diffusion, projection and torch."""
+    tau = 3.0 / max(dims) ** 2
+    g = torch.Generator(device="cuda").manual_seed(5)
+    A = torch.randn((9,) + dims, generator=g, device="cuda", dtype=torch.float64)
+    h = M.Mbo(dims, 3, tau, "f64")
+    h.project(A, A)
+    old, At, B = A.clone(), torch.empty_like(A), torch.empty_like(A)
+    h.diffuse(old, At)
+    h.project(At, B)
+    E = h.lyapunov(old)
+    rec = h.step(A, want_stats=True)
+    h.close()
+    det = lambda F: torch.linalg.det(F.reshape(3, 3, -1).permute(2, 0, 1))  # noqa: E731
+    assert rec["max_delta"] == float((A - old).abs().max())
+    assert rec["det_flips"] == int(((det(A) >= 0) != (det(old) >= 0)).sum())
+    assert rec["nonfinite"] == 0
+    assert rec["energy"] == pytest.approx(E, rel=1e-12)
+    s = torch.linalg.svdvals(At.reshape(3, 3, -1).permute(2, 0, 1))
+    clear = (s[:, 2] > 1e-6 * s[:, 0]) & (s[:, 1] + s[:, 2] > 1e-2)
+    assert float((A - B).abs().amax(0).reshape(-1)[clear].max()) <= 1e-12
