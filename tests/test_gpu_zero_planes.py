@@ -14,16 +14,18 @@ def M():
     return mbo
 
 
-def per_call(f, k=20):
+def per_call(calls, k=20):
+    """ms per call of each, the best of runs taken in turn."""
     e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
-    best = float("inf")
-    for _ in range(6):
-        e0.record()
-        for _ in range(k):
-            f()
-        e1.record()
-        e1.synchronize()
-        best = min(best, e0.elapsed_time(e1) / k)
+    best = [float("inf")] * len(calls)
+    for _ in range(10):
+        for i, f in enumerate(calls):
+            e0.record()
+            for _ in range(k):
+                f()
+            e1.record()
+            e1.synchronize()
+            best[i] = min(best[i], e0.elapsed_time(e1) / k)
     return best
 
 
@@ -36,7 +38,7 @@ def test_zero_channels_cost_no_more(M, dims, n):
     phases[0, ..., : dims[-1] // 2] = -1.0
     out = torch.empty_like(full)
     h = M.Mbo(dims, n, 3.0 / min(dims) ** 2, "f64")
-    t = [per_call(lambda: h.diffuse(a, out)) for a in (full, phases)]
+    t = per_call([lambda: h.diffuse(full, out), lambda: h.diffuse(phases, out)])
     # channels 2q and 2q + 1 share a plane: both zero
     zero = [c for c in range(n * n - 1) if c % 2 == 0 and not phases[c:c + 2].any()]
     for c in zero:
